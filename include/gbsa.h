@@ -123,8 +123,8 @@ typedef struct {
    * ISA either way. */
   uint32_t device_rounds;
   /* Order of the groups of equal names in the active list after round 0:
-   * 0 = the library chooses (the position order below whenever a round
-   * follows), 1 = ordered by each group's smallest member position, so that
+   * 0 = the library chooses (the position order below for large texts with
+   * many suffixes still active), 1 = ordered by each group's smallest member position, so that
    * groups of suffixes that move together (copies of a repeated text) sit
    * side by side and their partner-name reads share cache lines, 2 = rank
    * order (as round 0 leaves them). Same SA and ISA either way: a round

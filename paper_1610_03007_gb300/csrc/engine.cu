@@ -103,8 +103,10 @@ Layout make_layout(uint64_t N, uint32_t S) {
   L.bytehist = take(RADIX * 4);
   L.code = take(RADIX);
   L.segoff = take(((size_t)S + 1) * 4);
-  L.ka = take(Nm * 8);
-  L.kb = take(Nm * 8);
+  // The key buffers also hold the group order's scan sums and marks, which
+  // a batch of mostly empty texts needs more of than of keys.
+  L.ka = take(std::max<uint64_t>(Nm * 8, rank_sums_words(N + S, Nm / 2) * 4));
+  L.kb = take(std::max<uint64_t>(Nm * 8, rank_lines(N + S) * 32));
   L.va = take(Nm * 4);
   L.vb = take(Nm * 4);
   L.act0 = take(Nm * 8);
@@ -988,68 +990,62 @@ struct Build {
     return SA_OK;
   }
 
+  // Whether the groups are put in position order after round 0. It pays
+  // where the ISA (4 N bytes) is not held by the L2 anyway and enough
+  // suffixes stay active to repay the eight launches and the pass over the
+  // marks. Measured, position order against rank order: repeated Zipf
+  // 2^22 1.82 / 1.74 ms, 2^24 6.53 / 6.69, 2^26 25.6 / 30.8, 2^28 81.7 /
+  // 109.3; Markov DNA 2^24 2.29 / 2.21, 2^26 10.40 / 10.49, 2^28 26.3 / 29.9;
+  // words 2^26 11.50 / 11.48; with 1.5 % and 3 % active, DNA 2^26 5.38 /
+  // 5.30, Zipf bytes 2^26 7.29 / 7.20; below 2^22 about 0.07 ms more.
+  bool position_order_wanted(uint32_t m) const {
+    if (opt.group_order) return opt.group_order == 1;
+    return N >= (1ull << 24) && m >= N / 16;
+  }
+
   // The groups of the active list `cur` (hc: its counts) copied to the
   // other buffer set in order of their smallest member position, then
   // classified again (large groups, refine tile map); hc is re-read.
   sa_status reorder_groups(int cur, HostCtrl &hc) {
     const uint32_t G = hc.g_next(), m = hc.m_next();
     const int nxt = cur ^ 1;
-    const int sms = sm_count();
     // Buffers: the records go to the update queue (free now, 8 N bytes >=
-    // 16 G); after the sort only its order (the final value buffer) is
-    // needed, so both key buffers are free: the records in the new order
-    // go to one, the sizes and scan sums to the other.
-    uint4 *info = reinterpret_cast<uint4 *>(upd);
-    sa_status s = launch(SA_K_REORDER, 0, 8ull * m + 44ull * G, [&] {
-      return launch_group_minpos(act[cur], gstart[cur], gname[cur], ghead[cur], G, ka, va, info,
-                                 sms, st);
-    });
-    if (s != SA_OK) return s;
-    bytes += 8ull * m + 44ull * G;
-    // By the 32 position bits (constant digits skipped); the order is in the
-    // plan's final value buffer.
-    s = sort(G, spec_for(32));
-    if (s != SA_OK) return s;
-    uint4 *info_new = reinterpret_cast<uint4 *>(ka);
-    uint32_t *sizes = reinterpret_cast<uint32_t *>(kb);
-    uint32_t *sums = sizes + G;
-    if (2ull * G > N || inclusive_scan_sums_words(G) + G > 2ull * N) return SA_ERR_INTERNAL;
-    s = launch(SA_K_REORDER, 1, 40ull * G, [&] {
-      return launch_group_sizes(plan, info, G, info_new, sizes, ctrl, sms, st);
-    });
-    if (s != SA_OK) return s;
-    s = launch(SA_K_REORDER, 2, 8ull * G,
-               [&] { return launch_inclusive_scan(sizes, sizes, G, sums, st); });
-    if (s != SA_OK) return s;
+    // 16 G), the marks to a key buffer, the scan sums to the other.
     RegroupArgs ra{};
-    ra.info = info_new;
-    ra.act_in = act[cur];
-    ra.ends = sizes;
     ra.G = G;
     ra.m = m;
+    ra.positions = (uint32_t)std::min<uint64_t>(N + S, 0xFFFFFFFFull);
+    ra.act_in = act[cur];
+    ra.gstart_in = gstart[cur];
+    ra.gname_in = gname[cur];
+    ra.ghead_in = ghead[cur];
+    ra.lines = reinterpret_cast<uint32_t *>(kb);
+    ra.sums = reinterpret_cast<uint32_t *>(ka);
+    ra.info = reinterpret_cast<uint4 *>(upd);
     ra.act_out = act[nxt];
     ra.gstart_out = gstart[nxt];
     ra.gname_out = gname[nxt];
     ra.ghead_out = ghead[nxt];
     ra.ctrl = ctrl;
-    s = launch(SA_K_REORDER, 3, 16ull * m + 32ull * G,
-               [&] { return launch_regroup(ra, sms, st); });
+    if (2ull * G > N) return SA_ERR_INTERNAL;
+    const uint64_t rank_bytes = 68ull * G + 3 * 32ull * rank_lines(ra.positions);
+    sa_status s = launch(SA_K_REORDER, 0, rank_bytes,
+                         [&] { return launch_group_rank(ra, sm_count(), st); });
     if (s != SA_OK) return s;
-    bytes += 40ull * G + 8ull * G + 16ull * m + 32ull * G;
-    // Every group is now a "refine" group with its final name.
-    RoundCounts rc{};
-    rc.m_s = m;
-    rc.g_s = G;
-    CK(cudaMemcpyAsync(&ctrl->rc, &rc, sizeof(rc), cudaMemcpyHostToDevice, st));
+    launches += 4;
+    const uint64_t move_bytes = 48ull * G + 16ull * m;
+    s = launch(SA_K_REORDER, 1, move_bytes, [&] { return launch_regroup(ra, st); });
+    if (s != SA_OK) return s;
+    launches += 3;
+    bytes += rank_bytes + move_bytes;
     s = classify(nxt, G, 0);
     if (s != SA_OK) return s;
     HostCtrl h2{};
     s = read_ctrl(h2);
     if (s != SA_OK) return s;
-    const uint32_t passes = h2.passes;
-    s = flush(h2.pass_mask, 0);
+    s = flush(0, 0);
     if (s != SA_OK) return s;
-    bytes += (uint64_t)passes * 24 * G + 8ull * G;
+    bytes += 8ull * G;
     h2.passes = hc.passes;
     h2.pass_mask = hc.pass_mask;
     h2.upd = hc.upd;
@@ -1199,7 +1195,7 @@ struct Build {
       settle(hc);
     }
     if (want_trace) CK(cudaMemcpyAsync(opt.trace_isa, isa, N * 4, cudaMemcpyDeviceToDevice, st));
-    if (hc.m_next() > 0 && opt.group_order != 2) {
+    if (hc.m_next() > 0 && position_order_wanted(hc.m_next())) {
       // The later rounds read partner names through the ISA: groups in
       // position order make those reads of neighbouring groups neighbours.
       s = reorder_groups(cur, hc);

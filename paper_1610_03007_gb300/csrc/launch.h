@@ -315,29 +315,29 @@ cudaError_t launch_round_begin(const RoundBeginArgs &a, cudaStream_t stream);
 cudaError_t launch_round_end(const Ctrl *c, cudaGraphConditionalHandle loop, cudaStream_t stream);
 
 // ---- group order after round 0 (k_reorder.cu) -------------------------------
-// keys[g] = the smallest member position of group g, vals[g] = g,
-// info[g] = (start, size, name, head rank).
-cudaError_t launch_group_minpos(const uint64_t *act, const uint32_t *gstart, const uint32_t *gname,
-                                const uint32_t *ghead, uint32_t G, uint64_t *keys, uint32_t *vals,
-                                uint4 *info, int num_sms, cudaStream_t stream);
-// info_new[x] = info[plan->vfinal[x]], sizes[x] = its size.
-cudaError_t launch_group_sizes(const SortPlan *plan, const uint4 *info, uint32_t G,
-                               uint4 *info_new, uint32_t *sizes, Ctrl *ctrl, int num_sms,
-                               cudaStream_t stream);
-// out[i] = in[0] + .. + in[i] (may alias); sums: inclusive_scan_sums_words(m) words.
-cudaError_t launch_inclusive_scan(const uint32_t *in, uint32_t *out, uint64_t m, uint32_t *sums,
-                                  cudaStream_t stream);
-uint64_t inclusive_scan_sums_words(uint64_t m);
+// One line of marks: 7 words of bits and their predecessors' count.
+constexpr uint32_t RANK_LINE_BITS = 224;
+constexpr uint64_t rank_lines(uint64_t positions) { return positions / RANK_LINE_BITS + 1; }
+// Words of `sums` for a build of this many positions and at most N / 2 groups.
+constexpr uint64_t rank_sums_words(uint64_t positions, uint64_t groups) {
+  return (rank_lines(positions) > groups ? rank_lines(positions) : groups) / 2048 + 1;
+}
 struct RegroupArgs {
-  const uint4 *info;        // (start, size, name, head rank) of new group x
+  uint32_t G, m;            // groups and entries of the list
+  uint32_t positions;       // gapped positions (N + S)
   const uint64_t *act_in;   // entries in the old order
-  const uint32_t *ends;     // inclusive prefix sums of the sizes in the new order
-  uint32_t G, m;
+  const uint32_t *gstart_in, *gname_in, *ghead_in;  // G + 1, G, G entries
+  uint32_t *lines;          // rank_lines(positions) * 8 words
+  uint32_t *sums;           // rank_sums_words(positions, G) words
+  uint4 *info;              // G records (start, size, name, head rank) in the new order
   uint64_t *act_out;        // entries (x << 32) | i' in the new order
   uint32_t *gstart_out, *gname_out, *ghead_out;     // G + 1, G, G entries
-  Ctrl *ctrl;
+  Ctrl *ctrl;               // rc becomes (m, G) of the refine
 };
-cudaError_t launch_regroup(const RegroupArgs &a, int num_sms, cudaStream_t stream);
+// info[x] = the group with the x-th smallest first position.
+cudaError_t launch_group_rank(const RegroupArgs &a, int num_sms, cudaStream_t stream);
+// The tables and entries of the new order from info.
+cudaError_t launch_regroup(const RegroupArgs &a, cudaStream_t stream);
 
 // ---- position bucketing of ISA writes (k_bucket.cu) ------------------------
 constexpr uint32_t BUCKET_BLOCKS_MAX = 1024;
