@@ -83,6 +83,8 @@ struct Ctrl {
   RoundCounts rc;
   uint32_t zero[4];    // constant zeros (output offsets of round 0)
   uint32_t bucket_total;  // entries a translating position partition kept
+  uint32_t need_any;      // k_need_plan found granules that are not covered
+  uint32_t need_entries;  // entries k_need_collect wrote
   uint32_t tile_ctr[TILE_COUNTERS];  // one dynamic tile counter per launch
   RoundState rs;                     // device-driven rounds only
   RoundRecord rec[DEV_MAX_ROUNDS];
@@ -396,11 +398,11 @@ __device__ __forceinline__ uint32_t warp_rank_digit_match(uint32_t d, uint16_t *
   return before + __popc(peers & lt);
 }
 
-// Local index of gapped position ip: text s occupies the gapped positions
+// Text of gapped position ip: text s occupies the gapped positions
 // [seg_off[s] + s, seg_off[s+1] + s) (the slot after it is its end
 // sentinel), so gapped starts increase strictly even across empty texts.
-__device__ __forceinline__ uint32_t local_index(uint32_t ip, const uint32_t *seg_off, uint32_t S) {
-  if (S <= 1) return ip;
+__device__ __forceinline__ uint32_t gapped_segment(uint32_t ip, const uint32_t *seg_off,
+                                                   uint32_t S) {
   uint32_t lo = 0, hi = S - 1;  // the last s with seg_off[s] + s <= ip
   while (lo < hi) {
     const uint32_t mid = (lo + hi + 1) >> 1;
@@ -409,7 +411,14 @@ __device__ __forceinline__ uint32_t local_index(uint32_t ip, const uint32_t *seg
     else
       hi = mid - 1;
   }
-  return ip - (__ldg(seg_off + lo) + lo);
+  return lo;
+}
+
+// Local index of gapped position ip in its text.
+__device__ __forceinline__ uint32_t local_index(uint32_t ip, const uint32_t *seg_off, uint32_t S) {
+  if (S <= 1) return ip;
+  const uint32_t s = gapped_segment(ip, seg_off, S);
+  return ip - (__ldg(seg_off + s) + s);
 }
 
 // Inclusive warp scan.

@@ -29,6 +29,7 @@
 //   u32[N/2+1], large-group lists, the refine tile map, look-back status,
 //   control block, plan, histograms: about 67 bytes per character.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -81,11 +82,21 @@ struct NvtxRange {
 struct Layout {
   size_t ctrl, plan, hist, dbase, bytehist, code, segoff;
   size_t ka, kb, va, vb, act0, act1, upd, isa, gs0, gs1, gn0, gn1, gh0, gh1, gold;
-  size_t lg, loff, lbase, lold, tfirst, bcount, pm1;
+  size_t lg, loff, lbase, lold, tfirst, bcount, pm1, need;
   size_t st_sort, st_ren, total;
   size_t st_sort_bytes, st_ren_bytes;
-  uint32_t max_groups, max_large, max_tiles;
+  uint32_t max_groups, max_large, max_tiles, need_words;
 };
+
+// Granules of the needed ISA entries (k_isa.cu): position >> need_shift.
+uint32_t need_shift(uint64_t positions) {
+  uint32_t s = 0;
+  while (positions >> s >= (uint64_t)NEED_WORDS * 32) ++s;
+  return s;
+}
+uint32_t need_words(uint64_t positions) {
+  return (uint32_t)((positions >> need_shift(positions)) / 32 + 1);
+}
 
 Layout make_layout(uint64_t N, uint32_t S) {
   Layout L{};
@@ -128,6 +139,8 @@ Layout make_layout(uint64_t N, uint32_t S) {
   L.lold = take((size_t)L.max_large * 4);
   L.bcount = take((size_t)BUCKET_BLOCKS_MAX * RADIX * 4);
   L.pm1 = take(8);
+  L.need_words = need_words(N + S);
+  L.need = take(3 * (size_t)L.need_words * 4);
   L.max_tiles = (uint32_t)((Nm + REFINE_MIN_NOMINAL - 1) / REFINE_MIN_NOMINAL);
   L.tfirst = take(((size_t)L.max_tiles + 1) * 4);
   const uint64_t ts = std::max<uint64_t>(1, (N + SORT_TILE_MIN - 1) / SORT_TILE_MIN);
@@ -228,6 +241,91 @@ struct PinnedStage {
   }
 };
 
+// Costs of round 0's steps over all items in units of one radix pass, and
+// a pass's time: a fixed part and 7 ps per item (choose_split).
+constexpr double LOCAL_COST = 1.9, RENAME_COST = 1.5;
+constexpr double PASS_FIXED_US = 9.0, PASS_ITEM_US = 7e-6;
+// log2 of the bucket size that a tile takes about half of the time: buckets
+// of up to 512 items always fit, of 3072 and more never.
+constexpr double LOCAL_LARGE_LOG2 = 10.3;
+// From this length on, with at most a quarter of the suffixes active, the ISA gets only the entries that later rounds read
+// (k_isa.cu), and from the second on they go through a list that can be
+// bucketed by position (an ISA that the L2 holds is written directly).
+constexpr uint64_t NEED_MIN_N = 1ull << 22, COLLECT_MIN_N = 1ull << 25;
+// Texts at least this long wait for the gram histogram to model their
+// prefixes by its statistics; shorter ones take the character counts.
+constexpr uint64_t GRAM_MODEL_MIN = 1ull << 22;
+
+// How the probability of a k-character prefix is spread, as the normal
+// distribution of its logarithm over the text's positions: mean and variance
+// of -log2 p for the first g characters, then per further character (the
+// last of a g-character gram given the others). For choosing a sort only.
+struct PrefixModel {
+  // (and the least -log2 p, that of the most frequent prefix)
+  double g = 1, mean = 0, var = 0, mean1 = 0, var1 = 0, least = 0, least1 = 0;
+
+  static void moments(const double *p, const double *q, int n, double &mean, double &var,
+                      double &least) {
+    // of -log2 q under p
+    double s1 = 0, s2 = 0;
+    least = 64;
+    for (int i = 0; i < n; ++i)
+      if (p[i] > 0) {
+        const double x = -std::log2(q[i]);
+        s1 += p[i] * x;
+        s2 += p[i] * x * x;
+        least = std::min(least, x);
+      }
+    mean = s1;
+    var = std::max(0.0, s2 - s1 * s1);
+  }
+
+  static PrefixModel characters(const uint32_t *hist) {
+    double p[RADIX], total = 0;
+    for (int c = 0; c < RADIX; ++c) total += hist[c];
+    for (int c = 0; c < RADIX; ++c) p[c] = hist[c] / total;
+    PrefixModel m;
+    moments(p, p, RADIX, m.mean, m.var, m.least);
+    m.mean1 = m.mean;
+    m.var1 = m.var;
+    m.least1 = m.least;
+    return m;
+  }
+
+  // From the counts of the 8-bit grams of 8 / b characters.
+  static PrefixModel grams(const uint32_t *hist, uint32_t b) {
+    double p[RADIX], q[RADIX], total = 0;
+    for (int c = 0; c < RADIX; ++c) total += hist[c];
+    for (int c = 0; c < RADIX; ++c) p[c] = hist[c] / total;
+    const int last = 1 << b;
+    for (int c = 0; c < RADIX; c += last) {
+      double ctx = 0;
+      for (int x = 0; x < last; ++x) ctx += p[c + x];
+      for (int x = 0; x < last; ++x) q[c + x] = ctx > 0 ? p[c + x] / ctx : 0;
+    }
+    PrefixModel m;
+    m.g = 8.0 / b;
+    moments(p, p, RADIX, m.mean, m.var, m.least);
+    moments(p, q, RADIX, m.mean1, m.var1, m.least1);
+    return m;
+  }
+
+  // Share of a text of 2^log_len characters whose `chars`-character prefix
+  // occurs more than 2^log_large times.
+  double large_share(double chars, double log_len, double log_large) const {
+    if (chars <= 0) return log_len > log_large ? 1.0 : 0.0;
+    double mu = mean * chars / g, v = var * chars / g, top = least * chars / g;
+    if (chars > g) {
+      mu = mean + (chars - g) * mean1;
+      v = var + (chars - g) * var1;
+      top = least + (chars - g) * least1;
+    }
+    if (log_len - top < log_large - 1.0) return 0.0;
+    const double z = (log_large - (log_len - mu)) / std::sqrt(2.0 * std::max(v, 0.05));
+    return 0.5 * std::erfc(z);
+  }
+};
+
 struct HostCtrl {
   uint32_t error, err_where, passes, pass_mask;
   uint32_t m_s, g_s, m_l, g_l, upd, pad;
@@ -267,6 +365,8 @@ struct Build {
   uint32_t *ghead[2] = {nullptr, nullptr}, *gold = nullptr;
   uint32_t *lg = nullptr, *loff = nullptr, *lbase = nullptr, *lold = nullptr, *tfirst = nullptr;
   uint32_t *bcount = nullptr;  // position-bucketing counts (BUCKET_BLOCKS_MAX x 256)
+  uint32_t *need = nullptr;    // granules: active, covered, missing (k_isa.cu)
+  bool need_filtered = false;  // only needed ISA entries are written
   uint32_t *pm1 = nullptr;     // (passes, pass mask) of the first sort of an a-tuple round
   // launch bookkeeping
   uint32_t epoch = 0, slot = 0;
@@ -333,6 +433,7 @@ struct Build {
     lold = at<uint32_t>(L.lold);
     bcount = at<uint32_t>(L.bcount);
     pm1 = at<uint32_t>(L.pm1);
+    need = at<uint32_t>(L.need);
     tfirst = at<uint32_t>(L.tfirst);
     st_sort = at<uint64_t>(L.st_sort);
     st_ren = at<uint64_t>(L.st_ren);
@@ -431,8 +532,9 @@ struct Build {
   // passes are copied to pm1 afterwards; profile records tag pass + 32).
   // from_text (round 0, one text): pass 0 builds the keys from the text
   // (the pack wrote only the histograms), so it is kept even if constant.
+  // keep: further passes kept whatever their digits (launch_sort_plan).
   sa_status sort(uint32_t m, const DigitSpec &spec, bool hist_ready = false, int chain = 0,
-                 const PackArgs *from_text = nullptr) {
+                 const PackArgs *from_text = nullptr, uint32_t keep = 0) {
     sa_status s = SA_OK;
     if (!hist_ready) {
       CK(cudaMemsetAsync(hist, 0, (size_t)spec.P * RADIX * 4, st));
@@ -444,7 +546,7 @@ struct Build {
     }
     s = launch(SA_K_PLAN, 0, (uint64_t)spec.P * RADIX * 8, [&] {
       return launch_sort_plan(hist, dbase, spec, m, ka, kb, va, vb, plan, ctrl, st, nullptr,
-                              from_text != nullptr);
+                              keep | (from_text ? 1u : 0u));
     });
     if (s != SA_OK) return s;
     for (uint32_t p = 0; p < spec.P; ++p) {
@@ -481,6 +583,17 @@ struct Build {
     return SA_OK;
   }
 
+  // The top `digits` 8-bit digits of total_bits-bit keys.
+  static DigitSpec top_spec(uint32_t total_bits, uint32_t digits) {
+    DigitSpec s{};
+    s.P = digits;
+    for (uint32_t p = 0; p < digits; ++p) {
+      s.shift[p] = (uint8_t)(total_bits - (digits - p) * RADIX_BITS);
+      s.bits[p] = RADIX_BITS;
+    }
+    return s;
+  }
+
   static DigitSpec spec_for(uint32_t total_bits) {
     DigitSpec s{};
     s.P = (total_bits + RADIX_BITS - 1) / RADIX_BITS;
@@ -493,7 +606,7 @@ struct Build {
 
   // Rename of round 0 (all suffixes) or of the large groups of a later
   // round; writes the next active list at the device-side offsets `off_in`.
-  sa_status rename(uint32_t m, bool round0, uint32_t cb, uint32_t c0, uint32_t W,
+  sa_status rename(uint32_t m, uint32_t round0, uint32_t cb, uint32_t c0, uint32_t W,
                    const uint32_t *base_in, const uint32_t *old_in, uint32_t g_in, int out,
                    const uint32_t *off_in, bool wide = false) {
     RenameArgs ra{};
@@ -501,7 +614,7 @@ struct Build {
     ra.sec_buf[1] = wide ? kb : nullptr;
     ra.plan = plan;
     ra.m = m;
-    ra.round0 = round0 ? 1u : 0u;
+    ra.round0 = round0;
     ra.cb = cb;
     ra.c0 = c0;
     ra.seg_off = segoff;
@@ -593,7 +706,7 @@ struct Build {
     ba.blocks = std::min<uint32_t>(BUCKET_BLOCKS_MAX, 4 * sm_count());
     ba.counts = bcount;
     ba.out = kb;
-    ++(src_tag ? pend.bucket_surv : pend.bucket_upd);
+    if (src_tag != 4) ++(src_tag ? pend.bucket_surv : pend.bucket_upd);
     sa_status s = launch(SA_K_BUCKET, src_tag, PENDING,
                          [&] { return launch_bucket_count(ba, st); });
     if (s != SA_OK) return s;
@@ -629,17 +742,20 @@ struct Build {
       if (r.bytes != PENDING) continue;
       if (r.cls == SA_K_SCATTER) r.bytes = 12ull * hc.upd;
       if (r.cls == SA_K_APPLY) r.bytes = 12ull * hc.m_l;
-      if (r.cls == SA_K_BUCKET)
+      if (r.cls == SA_K_BUCKET && (r.pass & 4))
+        r.bytes = 0;
+      else if (r.cls == SA_K_BUCKET)
         r.bytes = ((r.pass & 1) ? 16ull : 8ull) * ((r.pass & 2) ? hc.m_l : hc.upd);
     }
   }
 
-  // Rename (round 0 or large groups) reads 12 bytes per item; writes 4
-  // (SA) + 8 (queued ISA entry) per unique item, 8 per survivor and 12 per
-  // surviving group (start, head rank, parent name).
-  static uint64_t rename_bytes(uint32_t m, uint32_t surv, uint32_t groups) {
+  // Rename (round 0 or large groups) reads 12 bytes per item; writes 4 (SA)
+  // and, after round 0, 8 (queued ISA entry) per unique item, 8 per survivor
+  // (and 4 of SA in round 0) and 12 per surviving group (start, head rank,
+  // parent name).
+  static uint64_t rename_bytes(uint32_t m, uint32_t surv, uint32_t groups, bool round0 = false) {
     const uint64_t u = m - surv;
-    return 12ull * m + 12 * u + 8ull * surv + 12ull * groups;
+    return 12ull * m + (round0 ? 4 : 12) * u + (round0 ? 12ull : 8ull) * surv + 12ull * groups;
   }
 
   // Refine: 8 bytes read and a - 1 4-byte gathers per item, 8 bytes of
@@ -1053,6 +1169,191 @@ struct Build {
     return SA_OK;
   }
 
+  // Round 0 after the radix sort of its keys' top `split` digits: the
+  // buckets of equal top bits tile by tile, those too large for a tile by
+  // the global sort and rename, then the classification. hc: the counts.
+  sa_status finish_buckets(int out, uint32_t split, uint32_t bits0, uint32_t cb, uint32_t c0,
+                           HostCtrl &hc) {
+    const uint32_t m = (uint32_t)N, R = bits0 - split * RADIX_BITS;
+    LocalArgs la{};
+    la.plan = plan;
+    la.m = m;
+    la.R = R;
+    la.cb = cb;
+    la.c0 = c0;
+    la.seg_off = segoff;
+    la.S = S;
+    la.N = m;
+    la.naming = naming;
+    la.isa_len = N + S + 1;
+    la.sa = sa;
+    la.act_out = act[out];
+    la.gstart_out = gstart[out];
+    la.gname_out = gname[out];
+    la.ghead_out = ghead[out];
+    la.upd = upd;
+    la.lg = lg;
+    la.loff = loff;
+    la.lbase = lbase;
+    la.lold = lold;
+    la.max_large = L.max_large;
+    la.max_groups = L.max_groups;
+    la.ctrl = ctrl;
+    sa_status s = launch(SA_K_RENAME, 0, 0, [&] { return launch_local(la, st); });
+    if (s != SA_OK) return s;
+    s = read_ctrl(hc);
+    if (s != SA_OK) return s;
+    const uint32_t mL = hc.m_large(), GL = hc.g_large(), passes = hc.passes;
+    if (hc.m_s > m || mL > m) return SA_ERR_INTERNAL;
+    // 12 bytes read and 4 written per item; 16 per survivor, 12 per group.
+    const uint64_t lb = 16ull * m + 16ull * hc.m_s + 12ull * hc.g_s;
+    bytes += (uint64_t)passes * 24 * m + lb;
+    s = flush(hc.pass_mask, lb);
+    if (s != SA_OK) return s;
+    if (hc.m_next() == 0 && mL == 0) return SA_OK;
+    if (mL > 0) {
+      // Every pass was kept, so the sorted keys are in A after an even
+      // number of them: the large buckets' items go to the other buffer.
+      const bool in_a = split % 2 == 0;
+      if (!in_a) std::swap(ka, kb), std::swap(va, vb);
+      GatherBigArgs ga{};
+      ga.kin = ka;
+      ga.vin = va;
+      ga.lg = lg;
+      ga.loff = loff;
+      ga.m = m;
+      ga.mL = mL;
+      ga.GL = GL;
+      ga.R = R;
+      ga.keys = kb;
+      ga.vals = vb;
+      ga.sa = sa;
+      ga.ctrl = ctrl;
+      s = launch(SA_K_GATHER, 0, 28ull * mL, [&] { return launch_gather_big(ga, st); });
+      std::swap(ka, kb), std::swap(va, vb);  // sort from the buffer just written
+      if (s == SA_OK) s = sort(mL, spec_for(R + (GL > 1 ? bits_for(GL - 1) : 0)));
+      if (in_a) std::swap(ka, kb), std::swap(va, vb);
+      if (s != SA_OK) return s;
+      s = rename(mL, 2, cb, c0, R, lbase, lold, GL, out, &ctrl->rc.m_s);
+      if (s != SA_OK) return s;
+      bytes += 28ull * mL;
+    }
+    CK(cudaMemsetAsync(&ctrl->rc.large, 0, sizeof(ctrl->rc.large), st));
+    const uint32_t g_cap = hc.g_s + mL / 2 + 1;
+    s = classify(out, g_cap, mL);
+    if (s != SA_OK) return s;
+    s = read_ctrl(hc);
+    if (s != SA_OK) return s;
+    const uint64_t rb = mL ? rename_bytes(mL, hc.m_l, hc.g_l, true) : 0;
+    settle(hc);
+    s = flush(hc.pass_mask, rb);
+    if (s != SA_OK) return s;
+    bytes += (mL ? (uint64_t)hc.passes * 24 * mL : 0) + rb + 8ull * g_cap;
+    hc.passes = passes + (mL ? hc.passes : 0);
+    return SA_OK;
+  }
+
+  // ISA entries of the final ranks in the SA: all, or those whose position
+  // is in `missing`. The list goes through the active buffer `buf`.
+  sa_status collect(int buf, const uint32_t *missing) {
+    CollectArgs ca{};
+    ca.sa = sa;
+    ca.N = (uint32_t)N;
+    ca.seg_off = segoff;
+    ca.S = S;
+    ca.shift = need_shift(N + S);
+    ca.words = L.need_words;
+    ca.missing = missing;
+    ca.out = act[buf];
+    ca.ctrl = ctrl;
+    CK(cudaMemsetAsync(&ctrl->need_entries, 0, 4, st));
+    sa_status s = launch(SA_K_SCATTER, 2, 4ull * N,
+                         [&] { return launch_need_collect(ca, sm_count(), st); });
+    if (s != SA_OK) return s;
+    bytes += 4ull * N;
+    const uint64_t *src = act[buf];
+    if (N >= COLLECT_MIN_N && N >= bucket_min) {
+      s = bucket(src, nullptr, &ctrl->need_entries, (uint32_t)N, 4);
+      if (s != SA_OK) return s;
+      src = kb;
+    }
+    uint32_t *ctr = nullptr, ep = 0;
+    s = next_launch(ctr, ep);
+    if (s != SA_OK) return s;
+    return launch(SA_K_SCATTER, 3, 0, [&] {
+      return launch_write_entries(src, &ctrl->need_entries, (uint32_t)N, isa, N + S + 1, ctr,
+                                  8 * sm_count(), st);
+    });
+  }
+
+  // The entries that rounds with partner offsets h, h * mult, .. read (all of
+  // them up to NEED_OFFSET_MAX for the first plan, else this round's), of the
+  // active list in buffer `from`.
+  sa_status fill_needed(int from, uint32_t m, uint64_t h, bool first) {
+    NeedArgs na{};
+    na.act = act[from];
+    na.m = m;
+    na.shift = need_shift(N + S);
+    for (uint64_t x = h; x <= N && na.offsets + mult <= NEED_OFFSETS; x *= mult) {
+      for (uint32_t j = 1; j < mult; ++j)
+        if (j * x <= N) na.h[na.offsets++] = (uint32_t)(j * x);
+      if (!first || x * mult > NEED_OFFSET_MAX) break;
+    }
+    na.words = L.need_words;
+    na.active = need;
+    na.covered = need + L.need_words;
+    na.missing = need + 2 * (size_t)L.need_words;
+    na.ctrl = ctrl;
+    CK(cudaMemsetAsync(&ctrl->need_any, 0, 4, st));
+    sa_status s = launch(SA_K_SCATTER, 4, 8ull * m,
+                         [&] { return launch_need_plan(na, sm_count(), st); });
+    if (s != SA_OK) return s;
+    ++launches;
+    bytes += 8ull * m;
+    return collect(from ^ 1, na.missing);
+  }
+
+  // Digits of the top that the radix sort of round 0 takes before the
+  // buckets are sorted tile by tile, or 0 for all digits: the cheapest by
+  // the model of the prefixes, in units of one pass over all items. A tile
+  // pass costs LOCAL_COST, the rename that it replaces RENAME_COST; items
+  // in buckets too large for a tile are gathered, sorted by the remaining
+  // digits and the bucket ordinal, and renamed.
+  uint32_t choose_split(const PrefixModel &model, uint32_t b, uint32_t segbits,
+                        uint32_t bits0) const {
+    const uint32_t P = (bits0 + RADIX_BITS - 1) / RADIX_BITS;
+#ifdef GBSA_SPLIT_PASSES
+    return std::min<uint32_t>(GBSA_SPLIT_PASSES, (bits0 - 1) / RADIX_BITS);
+#endif
+    double best = P + RENAME_COST;
+    uint32_t split = 0;
+    // Characters by the logarithm of their text's length.
+    double mass[33] = {};
+    for (uint32_t k = 0; k < S; ++k) {
+      const uint64_t len = off[k + 1] - off[k];
+      if (len) mass[bits_for(len) - 1] += (double)len / (double)N;
+    }
+    for (uint32_t p = 1; p * RADIX_BITS < bits0; ++p) {
+      const uint32_t T = p * RADIX_BITS;
+      const double chars = T > segbits ? (double)(T - segbits) / b : 0.0;
+      double big = 0.0;
+      for (int l = 0; l < 33; ++l)
+        if (mass[l] > 0.0) big += mass[l] * model.large_share(chars, l + 0.5, LOCAL_LARGE_LOG2);
+      const uint32_t R = bits0 - T;
+      double cost = p + LOCAL_COST;
+      if (big > 0.0) {  // its share of a pass, each with the fixed part of one
+        const double rest = (R + bits_for((uint64_t)(big * N / 4096.0)) + 7) / 8;
+        const double share = (big * N * PASS_ITEM_US + PASS_FIXED_US) / (N * PASS_ITEM_US + PASS_FIXED_US);
+        cost += share * (rest + 3.0 + RENAME_COST);
+      }
+      if (cost < best) {
+        best = cost;
+        split = p;
+      }
+    }
+    return split;
+  }
+
   void record(uint32_t r, uint32_t m, const HostCtrl &hc, uint32_t kbits) {
     if (!stats || r >= SA_MAX_ROUNDS) return;
     stats->active[r] = m;
@@ -1153,7 +1454,7 @@ struct Build {
     const uint32_t bits0 = cb + segbits;
     pk.spec = spec_for(bits0);
     pk.hist = hist;
-    pk.top_only = (S == 1 && 8 % b == 0 && cb % 8 == 0 && c0 <= 64 && pk.spec.P * 8 == cb) ? 1u : 0u;
+    pk.top_only = (S == 1 && 8 % b == 0 && cb % 8 == 0 && c0 <= 64) ? 1u : 0u;
     // One text with whole-character digits: the first radix pass forms the
     // keys from the text and the pack only counts (no packed copy written
     // and read back).
@@ -1162,33 +1463,72 @@ struct Build {
       pk.keys = nullptr;
       pk.vals = nullptr;
     }
+    // How many digits the radix sort takes before the buckets of equal top
+    // bits are sorted tile by tile (0: all of them, then the rename).
+    PrefixModel model = PrefixModel::characters(hh);
+    uint32_t split = 0;
+    if (!pk.top_only) {
+      split = choose_split(model, b, segbits, bits0);
+      if (split) pk.spec = top_spec(bits0, split);
+    }
     const uint64_t pack_bytes = keys_in_pass ? (uint64_t)N : 13ull * N;
-    CK(cudaMemsetAsync(hist, 0, (size_t)pk.spec.P * RADIX * 4, st));
+    CK(cudaMemsetAsync(hist, 0, (size_t)(pk.top_only ? MAX_PASSES : pk.spec.P) * RADIX * 4, st));
     s = launch(SA_K_PACK, 0, pack_bytes, [&] { return launch_pack(pk, st); });
     if (s != SA_OK) return s;
     bytes += pack_bytes;
+    if (pk.top_only) {
+      if (N >= GRAM_MODEL_MIN && b < 8) {
+        uint32_t grams[RADIX];
+        CK(fetch(grams, hist + (MAX_PASSES - 1) * RADIX, sizeof(grams)));
+        model = PrefixModel::grams(grams, b);
+      }
+      split = choose_split(model, b, segbits, bits0);
+      if (split) pk.spec = top_spec(bits0, split);
+      s = launch(SA_K_PACK, 1, 0, [&] { return launch_pack_fixup(pk, st); });
+      if (s != SA_OK) return s;
+    }
     inject_pending = opt.inject_stall != 0;
-    s = sort(N32, pk.spec, true, 0, keys_in_pass ? &pk : nullptr);
-    if (s != SA_OK) return s;
     int cur = 0;  // the active list, group starts and names of this round
-    s = rename(N32, true, cb, c0, 0, nullptr, nullptr, 0, cur, ctrl->zero);
-    if (s != SA_OK) return s;
-    s = classify(cur, N / 2 + 1, N32);
-    if (s != SA_OK) return s;
+    const bool want_trace = opt.trace_isa && opt.trace_cap > 0 && S == 1;
     HostCtrl hc{};
-    s = read_ctrl(hc);
-    if (s != SA_OK) return s;
     uint32_t m = N32;
-    const uint64_t rb0 = rename_bytes(m, hc.m_next(), hc.g_next());
-    settle(hc);
-    s = flush(hc.pass_mask, rb0);
+    s = sort(N32, pk.spec, true, 0, keys_in_pass ? &pk : nullptr, split ? 0xFFu : 0u);
     if (s != SA_OK) return s;
+    if (!split) {
+      s = rename(N32, 1, cb, c0, 0, nullptr, nullptr, 0, cur, ctrl->zero);
+      if (s != SA_OK) return s;
+      s = classify(cur, N / 2 + 1, N32);
+      if (s != SA_OK) return s;
+      s = read_ctrl(hc);
+      if (s != SA_OK) return s;
+      const uint64_t rb0 = rename_bytes(m, hc.m_next(), hc.g_next(), true);
+      settle(hc);
+      s = flush(hc.pass_mask, rb0);
+      if (s != SA_OK) return s;
+      bytes += (uint64_t)hc.passes * 24 * m + rb0;
+    } else {
+      s = finish_buckets(cur, split, bits0, cb, c0, hc);
+      if (s != SA_OK) return s;
+    }
     record(0, m, hc, bits0);
-    bytes += (uint64_t)hc.passes * 24 * m - (keys_in_pass ? 11ull * m : 0ull) + rb0;
+    bytes -= keys_in_pass ? 11ull * m : 0ull;
     // The unique suffixes' ISA entries are needed only by a later round, the
     // ISA output or the trace; a text resolved in round 0 skips them.
-    const bool want_trace = opt.trace_isa && opt.trace_cap > 0 && S == 1;
     if (hc.m_next() > 0 || isa_out || want_trace) {
+      need_filtered = !isa_out && !opt.trace_isa && !device_rounds_wanted() && N >= NEED_MIN_N &&
+                      hc.m_next() <= N / 4;
+      if (need_filtered) {
+        CK(cudaMemsetAsync(need, 0, 3 * (size_t)L.need_words * 4, st));
+        s = fill_needed(cur, hc.m_next(), c0, true);
+      } else if (N < COLLECT_MIN_N || bucket_min == 0xFFFFFFFFu) {
+        bytes += 8ull * N;
+        s = launch(SA_K_SCATTER, 1, 8ull * N, [&] {
+          return launch_isa_fill(sa, N32, segoff, S, isa, N + S + 1, st);
+        });
+      } else {
+        s = collect(cur ^ 1, nullptr);
+      }
+      if (s != SA_OK) return s;
       // Its records settle with round 0's counts, before round 1 reads new ones.
       s = scatter(hc.upd);
       if (s != SA_OK) return s;
@@ -1224,6 +1564,10 @@ struct Build {
       const uint32_t mL = hc.m_large(), GL = hc.g_large();
       const int nxt = cur ^ 1;
       CK(cudaMemsetAsync(&ctrl->rc, 0, sizeof(RoundCounts), st));
+      if (need_filtered && h > NEED_OFFSET_MAX) {  // beyond the first plan
+        s = fill_needed(cur, m, h, false);
+        if (s != SA_OK) return s;
+      }
       // Large groups: keys for the global radix sort (gathered before any
       // name of this round changes).
       uint32_t kbits = 0;
@@ -1313,7 +1657,7 @@ struct Build {
       s = launch(SA_K_REFINE, 0, 0, [&] { return launch_refine(rf, st); });
       if (s != SA_OK) return s;
       if (mL > 0) {
-        s = rename(mL, false, 0, 0, W, lbase, lold, GL, nxt, &ctrl->rc.m_s, mult > 2);
+        s = rename(mL, 0, 0, 0, W, lbase, lold, GL, nxt, &ctrl->rc.m_s, mult > 2);
         if (s != SA_OK) return s;
       }
       s = scatter(m);

@@ -165,8 +165,12 @@ __global__ void __launch_bounds__(PACK_BLOCK) k_pack(PackArgs a) {
     }
   }
   __syncthreads();
-  for (uint32_t x = a.top_only ? (a.spec.P - 1) * RADIX + tid : tid; x < a.spec.P * RADIX;
-       x += PACK_BLOCK) {
+  if (a.top_only) {
+    const uint32_t v = s_hist[a.spec.P - 1][tid];
+    if (v) atomicAdd(&a.hist[(MAX_PASSES - 1) * RADIX + tid], v);
+    return;
+  }
+  for (uint32_t x = tid; x < a.spec.P * RADIX; x += PACK_BLOCK) {
     const uint32_t v = (&s_hist[0][0])[x];
     if (v) atomicAdd(&a.hist[x], v);
   }
@@ -175,7 +179,7 @@ __global__ void __launch_bounds__(PACK_BLOCK) k_pack(PackArgs a) {
 // The digit histograms of a single text's keys from the top digit's alone,
 // when every digit covers g = 8 / b whole characters (b divides 8 and c0 * b
 // is a multiple of 8): digit p of the key at position i is the g-character
-// gram at i + q_p, q_p = (c0 * b - 8 (p + 1)) / b, with code 0 past the end
+// gram at i + q_p, q_p = (c0 * b - 8 - shift_p) / b, with code 0 past the end
 // of the text. Over i in [0, n) those grams are the grams at [q_p, n + q_p):
 // the top digit's histogram (q = 0, grams at [0, n)) minus the grams at
 // [0, q_p) plus q_p all-padding grams (digit 0). One block; q_p < 64.
@@ -185,7 +189,7 @@ __global__ void __launch_bounds__(RADIX) k_pack_hist_fixup(PackArgs a) {
   const uint32_t d = threadIdx.x;
   s_code[d] = a.code[d];
   const uint32_t P = a.spec.P, g = 8 / a.b;
-  const uint32_t top = a.hist[(P - 1) * RADIX + d];
+  const uint32_t top = a.hist[(MAX_PASSES - 1) * RADIX + d];
   __syncthreads();
   // grams at positions 0 .. 63 (all q_p are below c0 <= 64)
   if (d < 64) {
@@ -197,8 +201,8 @@ __global__ void __launch_bounds__(RADIX) k_pack_hist_fixup(PackArgs a) {
     s_gram[d] = v;
   }
   __syncthreads();
-  for (uint32_t p = 0; p + 1 < P; ++p) {
-    const uint32_t qp = (a.cb - 8 * (p + 1)) / a.b;
+  for (uint32_t p = 0; p < P; ++p) {
+    const uint32_t qp = (a.cb - 8 - a.spec.shift[p]) / a.b;
     uint32_t below = 0;
     for (uint32_t x = 0; x < qp; ++x) below += s_gram[x] == d ? 1u : 0u;
     a.hist[p * RADIX + d] = top - below + (d == 0 ? qp : 0u);
@@ -270,7 +274,7 @@ __global__ void __launch_bounds__(PACK_BLOCK) k_gram_hist(PackArgs a) {
   __syncthreads();
   uint32_t v = 0;
   for (int w = 0; w < PACK_BLOCK / 32; ++w) v += s_hist[w][tid];
-  if (v) atomicAdd(&a.hist[(a.spec.P - 1) * RADIX + tid], v);
+  if (v) atomicAdd(&a.hist[(MAX_PASSES - 1) * RADIX + tid], v);
 }
 
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream) {
@@ -288,9 +292,6 @@ cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream) {
       case 8: k_gram_hist<8><<<grid, PACK_BLOCK, 0, stream>>>(a); break;
       default: return cudaErrorInvalidValue;
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_pack_hist_fixup<<<1, RADIX, 0, stream>>>(a);
     return cudaGetLastError();
   }
   if (a.c0 >= PACK_SLIDE_MIN) {
@@ -300,8 +301,10 @@ cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream) {
     const uint64_t span = PACK_BLOCK * 8;
     k_pack<8><<<(unsigned)((a.N + span - 1) / span), PACK_BLOCK, 0, stream>>>(a);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !a.top_only) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pack_fixup(const PackArgs &a, cudaStream_t stream) {
   k_pack_hist_fixup<<<1, RADIX, 0, stream>>>(a);
   return cudaGetLastError();
 }

@@ -18,8 +18,9 @@
 //  - Unique (Algorithm 6): new_j differs from both neighbours, i.e.
 //    f_j and f_{j+1} (f_m = 1).
 //  - Discarding (Algorithm 5): a unique item is final: it writes SA[pos] = i
-//    and queues ISA[i] = pos (applied by k_scatter_updates when a later
-//    round or an output reads the ISA); the others are compacted, in order, into
+//    and, after rounds >= 1, queues ISA[i] = pos (applied by
+//    k_scatter_updates; after round 0 k_isa.cu takes the entries that a later
+//    round or an output reads from the SA); the others are compacted, in order, into
 //    the next active list with their group ordinal g', and each group's head
 //    records its start in that list, its head rank and its parent's name
 //    (the group's own name and the ISA entries of its members follow in
@@ -87,12 +88,13 @@ __device__ __forceinline__ bool rename_tile(RnSmem &S, const RenameArgs &a, cons
   const uint64_t *SEC = a.sec_buf[0] ? a.sec_buf[a.plan->final_idx ^ 1u] : nullptr;
   const uint32_t base = tile * RN_TILE;
   const uint32_t count = min((uint32_t)RN_TILE, m - base);
+  const bool first = a.round0 == 1;  // ranks are the sorted indices
 
   // Round 0: does the suffix at gapped position v (key k) have fewer than
   // c0 characters left in its text?
   auto tail = [&](uint64_t k, uint32_t v) -> bool {
     if (a.S <= 1) return a.N - v < a.c0;  // one text: gapped = plain positions
-    const uint32_t s = (uint32_t)(k >> a.cb);
+    const uint32_t s = a.round0 == 1 ? (uint32_t)(k >> a.cb) : gapped_segment(v, a.seg_off, a.S);
     const uint32_t off = __ldg(a.seg_off + s);
     const uint32_t len = __ldg(a.seg_off + s + 1) - off;
     return len - (v - (off + s)) < a.c0;
@@ -176,7 +178,7 @@ __device__ __forceinline__ bool rename_tile(RnSmem &S, const RenameArgs &a, cons
     if (lane < 2)
       status_store(a.status + (uint64_t)tile * 2 + lane,
                    status_word(epoch, tile == 0 ? ST_INC : ST_AGG, lane == 0 ? tot_s : tot_h));
-    if (lane == 2) S.upd_base = tot_u ? atomicAdd(&a.ctrl->rc.upd, tot_u) : 0u;
+    if (lane == 2) S.upd_base = tot_u && !a.round0 ? atomicAdd(&a.ctrl->rc.upd, tot_u) : 0u;
   }
   __syncthreads();
 
@@ -192,24 +194,27 @@ __device__ __forceinline__ bool rename_tile(RnSmem &S, const RenameArgs &a, cons
     const bool f = (fbits >> k) & 1u, fn = (fnbits >> k) & 1u;
     const bool uniq = valid && f && fn;
     const uint32_t U = __ballot_sync(0xffffffffu, uniq);
+    if (first && valid && !uniq && base + e < a.N) a.sa[base + e] = SA_NONE;
     if (!uniq) continue;
     const uint32_t j = base + e, ip = val[k];
-    const uint32_t g = a.round0 ? 0u : (uint32_t)(key[k] >> a.W);
-    if (!a.round0 && g >= g_in) {  // never taken unless a logic error
+    const uint32_t g = first ? 0u : (uint32_t)(key[k] >> a.W);
+    if (!first && g >= g_in) {  // never taken unless a logic error
       raise_error(a.ctrl, ERR_INTERNAL, 4);
       continue;
     }
-    const uint32_t head = a.round0 ? j : __ldg(a.base_in + g) + j;
+    const uint32_t head = first ? j : __ldg(a.base_in + g) + j;
     if (head >= a.N || ip >= a.isa_len) {  // never taken unless a logic error
       raise_error(a.ctrl, ERR_INTERNAL, 3);
       continue;
     }
-    const uint32_t slot = S.upd_base + (uint32_t)(S.pre[k * RN_WARPS + warp] & 0x1FFFFFu) +
-                          __popc(U & lt);
-    a.upd[slot] = ((uint64_t)head << 32) | ip;
+    if (!a.round0) {
+      const uint32_t slot = S.upd_base + (uint32_t)(S.pre[k * RN_WARPS + warp] & 0x1FFFFFu) +
+                            __popc(U & lt);
+      a.upd[slot] = ((uint64_t)head << 32) | ip;
+    }
     uint32_t local = ip;
     if (a.S > 1) {
-      if (a.round0) {
+      if (first) {
         const uint32_t s = (uint32_t)(key[k] >> a.cb);
         local = ip - (__ldg(a.seg_off + s) + s);
       } else {
@@ -270,19 +275,19 @@ __device__ __forceinline__ bool rename_tile(RnSmem &S, const RenameArgs &a, cons
     a.act_out[surv0 + sidx] = ((uint64_t)ord << 32) | ip;
     if (f) {  // the head of a surviving group
       const uint32_t j = base + e;
-      const uint32_t g = a.round0 ? 0u : (uint32_t)(key[k] >> a.W);
-      if (!a.round0 && g >= g_in) {  // never taken unless a logic error
+      const uint32_t g = first ? 0u : (uint32_t)(key[k] >> a.W);
+      if (!first && g >= g_in) {  // never taken unless a logic error
         raise_error(a.ctrl, ERR_INTERNAL, 4);
         continue;
       }
-      const uint32_t head = a.round0 ? j : __ldg(a.base_in + g) + j;
+      const uint32_t head = first ? j : __ldg(a.base_in + g) + j;
       if (head >= a.N) {  // never taken unless a logic error
         raise_error(a.ctrl, ERR_INTERNAL, 3);
         continue;
       }
       a.gstart_out[ord] = surv0 + sidx;
       a.ghead_out[ord] = head;
-      a.gold_out[ord] = a.round0 ? NO_NAME : __ldg(a.old_in + g);
+      a.gold_out[ord] = first ? NO_NAME : __ldg(a.old_in + g);
     }
   }
   return true;

@@ -88,7 +88,7 @@ constexpr float MATCH_RANK_MAX_DISTINCT = 24.f;
 __global__ void __launch_bounds__(RADIX)
 k_sort_plan(const uint32_t *__restrict__ hist, uint32_t *__restrict__ digit_base, DigitSpec spec,
             uint32_t m, uint64_t *ka, uint64_t *kb, uint32_t *va, uint32_t *vb,
-            SortPlan *plan, Ctrl *ctrl, const RoundState *rs, uint32_t keep_first) {
+            SortPlan *plan, Ctrl *ctrl, const RoundState *rs, uint32_t keep) {
   __shared__ uint32_t s_tmp[RADIX / 32 + 1];
   if (rs) {  // device-driven rounds
     if (!rs->live) return;
@@ -107,7 +107,7 @@ k_sort_plan(const uint32_t *__restrict__ hist, uint32_t *__restrict__ digit_base
     digit_base[p * RADIX + d] = excl;
     // A digit position is constant iff one bin holds every key.
     const int constant = __syncthreads_or(c == m);
-    if (d == 0) s_active[p] = constant && !(keep_first && p == 0) ? 0u : 1u;
+    if (d == 0) s_active[p] = constant && !((keep >> p) & 1u) ? 0u : 1u;
     // Expected distinct digits among 32 keys drawn from this histogram:
     // sum over d of 1 - (1 - p_d)^32. Few (a skewed alphabet) -> the pass
     // ranks with match.any, else with the shared-memory masks.
@@ -160,9 +160,9 @@ k_sort_plan(const uint32_t *__restrict__ hist, uint32_t *__restrict__ digit_base
 cudaError_t launch_sort_plan(const uint32_t *hist, uint32_t *digit_base, const DigitSpec &spec,
                              uint32_t m, uint64_t *ka, uint64_t *kb, uint32_t *va,
                              uint32_t *vb, SortPlan *plan, Ctrl *ctrl, cudaStream_t stream,
-                             const RoundState *rs, bool keep_first) {
+                             const RoundState *rs, uint32_t keep) {
   k_sort_plan<<<1, RADIX, 0, stream>>>(hist, digit_base, spec, m, ka, kb, va, vb, plan, ctrl, rs,
-                                       keep_first ? 1u : 0u);
+                                       keep);
   return cudaGetLastError();
 }
 

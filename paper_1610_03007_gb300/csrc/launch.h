@@ -56,13 +56,16 @@ struct PackArgs {
   DigitSpec spec;          // digits of the following radix sort
   uint32_t *hist;          // out: += their histograms (P * 256, zeroed by the caller)
   // 1: one text whose digits hold whole characters (b divides 8, cb a
-  // multiple of 8, P = cb / 8): only the top digit is counted per key and
-  // the other histograms are derived from it (k_pack_hist_fixup).
+  // multiple of 8): only the top digit is counted per key and the other
+  // histograms are derived from it (launch_pack_fixup).
   uint32_t top_only;
 };
-// keys == NULL (top_only only): the histograms alone (the first radix pass
-// then builds the keys from the text, PassArgs.text).
+// keys == NULL (top_only only): only the top digit's histogram (the first
+// radix pass then builds the keys from the text, PassArgs.text). With
+// top_only the counts go to the last of the MAX_PASSES rows, from which
+// launch_pack_fixup derives the rows of the digits in spec.
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream);
+cudaError_t launch_pack_fixup(const PackArgs &a, cudaStream_t stream);
 
 // ---- step A2: radix sort (k_sort.cu) ------------------------------------
 // hist[P*256] += digit counts of keys[0, m) for the digits in spec.
@@ -72,12 +75,13 @@ cudaError_t launch_digit_histogram(const uint64_t *keys, uint32_t m, const Digit
                                    uint32_t *hist, int num_sms, cudaStream_t stream,
                                    const RoundState *rs = nullptr);
 // Exclusive digit offsets, constant-digit skipping and buffer ping-pong.
-// keep_first: pass 0 is kept even if its digit is constant (it is the pass
-// that reads the text, PassArgs.text).
+// keep: bit p keeps pass p even if its digit is constant (the pass that
+// reads the text, PassArgs.text; every pass, so that the host knows which
+// buffer the result is in).
 cudaError_t launch_sort_plan(const uint32_t *hist, uint32_t *digit_base, const DigitSpec &spec,
                              uint32_t m, uint64_t *ka, uint64_t *kb, uint32_t *va,
                              uint32_t *vb, SortPlan *plan, Ctrl *ctrl, cudaStream_t stream,
-                             const RoundState *rs = nullptr, bool keep_first = false);
+                             const RoundState *rs = nullptr, uint32_t keep = 0);
 // One stable one-sweep pass over digit p of the plan.
 struct PassArgs {
   const SortPlan *plan;
@@ -115,7 +119,10 @@ cudaError_t launch_copy_back(const SortPlan *plan, uint64_t *ka, uint32_t *va, u
 struct RenameArgs {
   const SortPlan *plan;      // sorted keys / gapped positions
   uint32_t m;
-  uint32_t round0;           // 1: initial naming with the end-of-text rules
+  // 1: initial naming with the end-of-text rules; 2: the same for the
+  // buckets k_local left to the global path (keys (bucket << W) | low bits,
+  // ranks from base_in).
+  uint32_t round0;
   uint32_t cb;               // round 0: segment id = key >> cb (cb < 64)
   uint32_t c0;               // round 0: characters per key
   const uint32_t *seg_off;   // S+1 ungapped offsets
@@ -127,11 +134,14 @@ struct RenameArgs {
   const uint32_t *base_in;   // later rounds: head rank - start of group g
   const uint32_t *old_in;    // later rounds: name of group g (round 0: NULL)
   uint32_t g_in;             // later rounds: groups in base_in (bounds guard)
-  uint64_t *upd;             // queued ISA entries (head << 32 | i') of new unique suffixes
+  // Queued ISA entries (head << 32 | i') of new unique suffixes; in round 0
+  // (round0 != 0) none: k_isa.cu takes them from the SA.
+  uint64_t *upd;
   uint32_t *isa;             // gapped ISA (not written; bounds of gapped positions)
   uint64_t isa_len;          // entries of isa (bounds guard)
   uint32_t N;                // total characters = entries of sa (bounds guard)
   uint32_t *sa;              // SA, written with indices local to each text
+                             // (round0 = 1: SA_NONE at the survivors' ranks)
   uint64_t *act_out;         // survivors: (g' << 32) | i'
   uint32_t *gstart_out;      // start of each surviving group in act_out
   uint32_t *ghead_out;       // head rank (SA interval start) of each surviving group
@@ -153,6 +163,71 @@ struct RenameArgs {
 #endif
 constexpr int RENAME_TILE = 256 * GBSA_RN_ITEMS;
 cudaError_t launch_rename(const RenameArgs &a, cudaStream_t stream);
+
+// ---- round 0 by buckets of equal top bits (k_local.cu) -------------------
+constexpr uint32_t SA_NONE = 0xFFFFFFFFu;  // SA entry of a rank that is not final
+constexpr int LOCAL_TILE = 2560;           // window of one tile
+struct LocalArgs {
+  const SortPlan *plan;     // keys sorted by the bits from R up / gapped positions
+  uint32_t m, R;
+  uint32_t cb, c0;          // as RenameArgs
+  const uint32_t *seg_off;
+  uint32_t S, N;
+  uint32_t naming;
+  uint64_t isa_len;
+  uint32_t *sa;             // unique suffixes at their ranks, SA_NONE elsewhere
+  uint64_t *act_out;        // survivors of the tiles' buckets, as the refine's
+  uint32_t *gstart_out, *gname_out, *ghead_out;
+  uint64_t *upd;            // (name << 32) | i' of every survivor
+  // Buckets too large for a tile: start, start among their items, start
+  // less that, NO_NAME; rc.large counts them (buckets << 32 | items).
+  uint32_t *lg, *loff, *lbase, *lold;
+  uint32_t max_large, max_groups;
+  Ctrl *ctrl;               // rc.m_s / rc.g_s / rc.upd reserve the outputs
+};
+cudaError_t launch_local(const LocalArgs &a, cudaStream_t stream);
+struct GatherBigArgs {
+  const uint64_t *kin;      // the sorted keys and positions k_local read
+  const uint32_t *vin;
+  const uint32_t *lg, *loff;
+  uint32_t m, mL, GL, R;
+  uint64_t *keys;           // (bucket << R) | low bits of the key
+  uint32_t *vals;
+  uint32_t *sa;             // SA_NONE at the buckets' ranks
+  Ctrl *ctrl;
+};
+cudaError_t launch_gather_big(const GatherBigArgs &a, cudaStream_t stream);
+
+// ---- ISA entries of the suffixes final after round 0 (k_isa.cu) ------------
+// ISA[i'] = j for every rank j whose SA entry is not SA_NONE.
+cudaError_t launch_isa_fill(const uint32_t *sa, uint32_t N, const uint32_t *seg_off, uint32_t S,
+                            uint32_t *isa, uint64_t isa_len, cudaStream_t stream);
+
+constexpr uint32_t NEED_WORDS = 1u << 21;        // 2^26 granules
+constexpr uint32_t NEED_OFFSETS = 64;
+constexpr uint64_t NEED_OFFSET_MAX = 1ull << 17; // rounds the first plan covers
+struct NeedArgs {
+  const uint64_t *act;  // active entries (their low words are positions)
+  uint32_t m;
+  uint32_t shift;       // granule of a position: position >> shift
+  uint32_t words;       // words of bits in use
+  uint32_t offsets;     // partner offsets of the rounds planned for
+  uint32_t h[NEED_OFFSETS];
+  uint32_t *active, *covered, *missing;  // `words` each
+  Ctrl *ctrl;           // need_any is set when a granule is missing
+};
+cudaError_t launch_need_plan(const NeedArgs &a, int num_sms, cudaStream_t stream);
+struct CollectArgs {
+  const uint32_t *sa;
+  uint32_t N;
+  const uint32_t *seg_off;
+  uint32_t S;
+  uint32_t shift, words;    // as NeedArgs
+  const uint32_t *missing;  // NULL: every final rank
+  uint64_t *out;            // (rank << 32) | i', ctrl->need_entries of them (N at most)
+  Ctrl *ctrl;
+};
+cudaError_t launch_need_collect(const CollectArgs &a, int num_sms, cudaStream_t stream);
 
 // ---- rounds >= 1: small-group refine and large-group path (k_refine.cu) --
 // Groups of up to REFINE_SMALL_MAX members are refined inside one tile
@@ -294,6 +369,12 @@ cudaError_t launch_scatter_updates(const uint64_t *upd, uint32_t max_upd, uint32
                                    uint64_t isa_len, Ctrl *ctrl, cudaStream_t stream,
                                    const uint64_t *bucketed = nullptr,
                                    const RoundState *rs = nullptr, uint32_t grid_cap = 0);
+
+// ISA[i'] = name for entries[0, min(*count, max_count)) = (name << 32) | i',
+// by at most grid_cap blocks.
+cudaError_t launch_write_entries(const uint64_t *entries, const uint32_t *count,
+                                 uint32_t max_count, uint32_t *isa, uint64_t isa_len,
+                                 uint32_t *tile_ctr, uint32_t grid_cap, cudaStream_t stream);
 
 // ---- device-driven rounds (k_rounds.cu) ------------------------------------
 // Look-back epochs one device-driven round may use (its launches take the
