@@ -83,6 +83,7 @@ struct Ctrl {
   RoundCounts rc;
   uint32_t zero[4];    // constant zeros (output offsets of round 0)
   uint32_t bucket_total;  // entries a translating position partition kept
+  uint32_t done[2];       // finished blocks of the kernels whose last one reports to the host
   uint32_t need_any;      // k_need_plan found granules that are not covered
   uint32_t need_entries;  // entries k_need_collect wrote
   uint32_t tile_ctr[TILE_COUNTERS];  // one dynamic tile counter per launch

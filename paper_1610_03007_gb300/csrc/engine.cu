@@ -83,8 +83,7 @@ struct Layout {
   size_t ctrl, plan, hist, dbase, bytehist, code, segoff;
   size_t ka, kb, va, vb, act0, act1, upd, isa, gs0, gs1, gn0, gn1, gh0, gh1, gold;
   size_t lg, loff, lbase, lold, tfirst, bcount, pm1, need;
-  size_t st_sort, st_ren, total;
-  size_t st_sort_bytes, st_ren_bytes;
+  size_t st_sort, st_ren, zeroed, total;
   uint32_t max_groups, max_large, max_tiles, need_words;
 };
 
@@ -107,11 +106,18 @@ Layout make_layout(uint64_t N, uint32_t S) {
     return r;
   };
   const uint64_t Nm = N ? N : 1;
+  // What starts at zero, in one piece: control block, histograms and the
+  // look-back status words.
   L.ctrl = take(sizeof(Ctrl));
-  L.plan = take(sizeof(SortPlan));
   L.hist = take(MAX_PASSES * RADIX * 4);
-  L.dbase = take(MAX_PASSES * RADIX * 4);
   L.bytehist = take(RADIX * 4);
+  const uint64_t ts = std::max<uint64_t>(1, (N + SORT_TILE_MIN - 1) / SORT_TILE_MIN);
+  L.st_sort = take(ts * RADIX * 8);
+  const uint64_t tr = std::max<uint64_t>(1, (N + RENAME_TILE - 1) / RENAME_TILE);
+  L.st_ren = take(tr * 3 * 8);
+  L.zeroed = o;
+  L.plan = take(sizeof(SortPlan));
+  L.dbase = take(MAX_PASSES * RADIX * 4);
   L.code = take(RADIX);
   L.segoff = take(((size_t)S + 1) * 4);
   // The key buffers also hold the group order's scan sums and marks, which
@@ -143,12 +149,6 @@ Layout make_layout(uint64_t N, uint32_t S) {
   L.need = take(3 * (size_t)L.need_words * 4);
   L.max_tiles = (uint32_t)((Nm + REFINE_MIN_NOMINAL - 1) / REFINE_MIN_NOMINAL);
   L.tfirst = take(((size_t)L.max_tiles + 1) * 4);
-  const uint64_t ts = std::max<uint64_t>(1, (N + SORT_TILE_MIN - 1) / SORT_TILE_MIN);
-  L.st_sort_bytes = ts * RADIX * 8;
-  L.st_sort = take(L.st_sort_bytes);
-  const uint64_t tr = std::max<uint64_t>(1, (N + RENAME_TILE - 1) / RENAME_TILE);
-  L.st_ren_bytes = tr * 3 * 8;
-  L.st_ren = take(L.st_ren_bytes);
   L.total = o;
   return L;
 }
@@ -366,6 +366,7 @@ struct Build {
   uint32_t *lg = nullptr, *loff = nullptr, *lbase = nullptr, *lold = nullptr, *tfirst = nullptr;
   uint32_t *bcount = nullptr;  // position-bucketing counts (BUCKET_BLOCKS_MAX x 256)
   uint32_t *need = nullptr;    // granules: active, covered, missing (k_isa.cu)
+  bool isa_cleared = false;
   bool need_filtered = false;  // only needed ISA entries are written
   uint32_t *pm1 = nullptr;     // (passes, pass mask) of the first sort of an a-tuple round
   // launch bookkeeping
@@ -521,6 +522,10 @@ struct Build {
 
   sa_status read_ctrl(HostCtrl &hc) {
     CK(fetch(&hc, ctrl, sizeof(HostCtrl)));
+    return ctrl_status(hc);
+  }
+
+  static sa_status ctrl_status(const HostCtrl &hc) {
     if (hc.error == ERR_TIMEOUT) return SA_ERR_TIMEOUT;
     if (hc.error != ERR_NONE) return SA_ERR_INTERNAL;
     return SA_OK;
@@ -534,7 +539,8 @@ struct Build {
   // (the pack wrote only the histograms), so it is kept even if constant.
   // keep: further passes kept whatever their digits (launch_sort_plan).
   sa_status sort(uint32_t m, const DigitSpec &spec, bool hist_ready = false, int chain = 0,
-                 const PackArgs *from_text = nullptr, uint32_t keep = 0) {
+                 const PackArgs *from_text = nullptr, uint32_t keep = 0,
+                 const PackArgs *grams = nullptr) {
     sa_status s = SA_OK;
     if (!hist_ready) {
       CK(cudaMemsetAsync(hist, 0, (size_t)spec.P * RADIX * 4, st));
@@ -546,7 +552,7 @@ struct Build {
     }
     s = launch(SA_K_PLAN, 0, (uint64_t)spec.P * RADIX * 8, [&] {
       return launch_sort_plan(hist, dbase, spec, m, ka, kb, va, vb, plan, ctrl, st, nullptr,
-                              keep | (from_text ? 1u : 0u));
+                              keep | (from_text ? 1u : 0u), grams);
     });
     if (s != SA_OK) return s;
     for (uint32_t p = 0; p < spec.P; ++p) {
@@ -1169,6 +1175,15 @@ struct Build {
     return SA_OK;
   }
 
+  // The ISA starts all-ones, so that every end slot reads as the sentinel;
+  // once per build, before its first entry (a text that round 0 resolves
+  // writes none).
+  sa_status clear_isa() {
+    if (!isa_cleared) CK(cudaMemsetAsync(isa, 0xFF, (N + S + 1) * 4, st));
+    isa_cleared = true;
+    return SA_OK;
+  }
+
   // Round 0 after the radix sort of its keys' top `split` digits: the
   // buckets of equal top bits tile by tile, those too large for a tile by
   // the global sort and rename, then the classification. hc: the counts.
@@ -1199,9 +1214,16 @@ struct Build {
     la.max_large = L.max_large;
     la.max_groups = L.max_groups;
     la.ctrl = ctrl;
+    if (stage_readbacks) la.host = reinterpret_cast<uint32_t *>(stage.p);
     sa_status s = launch(SA_K_RENAME, 0, 0, [&] { return launch_local(la, st); });
     if (s != SA_OK) return s;
-    s = read_ctrl(hc);
+    if (la.host) {
+      CK(cudaStreamSynchronize(st));
+      memcpy(&hc, stage.p, sizeof(hc));
+      s = ctrl_status(hc);
+    } else {
+      s = read_ctrl(hc);
+    }
     if (s != SA_OK) return s;
     const uint32_t mL = hc.m_large(), GL = hc.g_large(), passes = hc.passes;
     if (hc.m_s > m || mL > m) return SA_ERR_INTERNAL;
@@ -1238,6 +1260,8 @@ struct Build {
       if (s != SA_OK) return s;
       bytes += 28ull * mL;
     }
+    s = clear_isa();
+    if (s != SA_OK) return s;
     CK(cudaMemsetAsync(&ctrl->rc.large, 0, sizeof(ctrl->rc.large), st));
     const uint32_t g_cap = hc.g_s + mL / 2 + 1;
     s = classify(out, g_cap, mL);
@@ -1372,30 +1396,37 @@ struct Build {
     prof = opt.profile != 0 && stats != nullptr;
     naming = opt.paper_names ? NAMES_HEAD : NAMES_RETAIN;
     mult = opt.multiplier ? opt.multiplier : 2;  // checked by the entry points
-    // Clear what must start at zero; the ISA starts all-ones so every end
-    // slot reads as the sentinel.
-    CK(cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), st));
-    CK(cudaMemsetAsync(st_sort, 0, L.st_sort_bytes, st));
-    CK(cudaMemsetAsync(st_ren, 0, L.st_ren_bytes, st));
-    CK(cudaMemsetAsync(bytehist, 0, RADIX * 4, st));
-    CK(cudaMemsetAsync(isa, 0xFF, (N + S + 1) * 4, st));
-    CK(cudaMemcpyAsync(segoff, off.data(), ((size_t)S + 1) * 4, cudaMemcpyHostToDevice, st));
+    CK(cudaMemsetAsync(ws, 0, L.zeroed, st));
+    if (S > 1)
+      CK(cudaMemcpyAsync(segoff, off.data(), ((size_t)S + 1) * 4, cudaMemcpyHostToDevice, st));
 
     // ---- A0: alphabet ----
-    sa_status s = launch(SA_K_BYTE_HIST, 0, N, [&] {
-      return launch_byte_histogram(text, N, bytehist, sm_count(), st);
-    });
+    if (stage_readbacks && stage.get() != cudaSuccess) {
+      cudaGetLastError();  // no pinned block to be had: the copy engine instead
+      stage_readbacks = false;
+    }
+    AlphabetArgs aa{};
+    aa.text = text;
+    aa.n = N;
+    aa.hist = bytehist;
+    aa.done = &ctrl->done[0];
+    aa.code = code;
+    aa.seg_off = S == 1 ? segoff : nullptr;
+    aa.host = stage_readbacks ? reinterpret_cast<uint32_t *>(stage.p) : nullptr;
+    sa_status s =
+        launch(SA_K_BYTE_HIST, 0, N, [&] { return launch_byte_histogram(aa, sm_count(), st); });
     if (s != SA_OK) return s;
     uint32_t hh[RADIX];
-    CK(fetch(hh, bytehist, sizeof(hh)));
+    if (aa.host) {
+      CK(cudaStreamSynchronize(st));
+      memcpy(hh, stage.p, sizeof(hh));
+    } else {
+      CK(fetch(hh, bytehist, sizeof(hh)));
+    }
     s = flush(0, 0);
     if (s != SA_OK) return s;
-    uint8_t hcode[RADIX];
     uint32_t sigma = 0;
-    for (int c = 0; c < RADIX; ++c) {
-      hcode[c] = (uint8_t)sigma;  // order-preserving dense code
-      if (hh[c]) ++sigma;
-    }
+    for (int c = 0; c < RADIX; ++c) sigma += hh[c] ? 1u : 0u;
     const uint32_t b = std::max<uint32_t>(1, bits_for(sigma - 1));
     const uint32_t segbits = S > 1 ? bits_for(S - 1) : 0;
     // Parameters: the caller's options, else the tuning table's entry for
@@ -1425,7 +1456,6 @@ struct Build {
     uint32_t c0 = (64 - segbits) / b;
     if (h0) c0 = std::min(c0, h0);
     const uint32_t cb = c0 * b;
-    CK(cudaMemcpyAsync(code, hcode, sizeof(hcode), cudaMemcpyHostToDevice, st));
     bytes += N;
     if (stats) {
       stats->sigma = sigma;
@@ -1472,7 +1502,6 @@ struct Build {
       if (split) pk.spec = top_spec(bits0, split);
     }
     const uint64_t pack_bytes = keys_in_pass ? (uint64_t)N : 13ull * N;
-    CK(cudaMemsetAsync(hist, 0, (size_t)(pk.top_only ? MAX_PASSES : pk.spec.P) * RADIX * 4, st));
     s = launch(SA_K_PACK, 0, pack_bytes, [&] { return launch_pack(pk, st); });
     if (s != SA_OK) return s;
     bytes += pack_bytes;
@@ -1484,17 +1513,18 @@ struct Build {
       }
       split = choose_split(model, b, segbits, bits0);
       if (split) pk.spec = top_spec(bits0, split);
-      s = launch(SA_K_PACK, 1, 0, [&] { return launch_pack_fixup(pk, st); });
-      if (s != SA_OK) return s;
     }
     inject_pending = opt.inject_stall != 0;
     int cur = 0;  // the active list, group starts and names of this round
     const bool want_trace = opt.trace_isa && opt.trace_cap > 0 && S == 1;
     HostCtrl hc{};
     uint32_t m = N32;
-    s = sort(N32, pk.spec, true, 0, keys_in_pass ? &pk : nullptr, split ? 0xFFu : 0u);
+    s = sort(N32, pk.spec, true, 0, keys_in_pass ? &pk : nullptr, split ? 0xFFu : 0u,
+             pk.top_only ? &pk : nullptr);
     if (s != SA_OK) return s;
     if (!split) {
+      s = clear_isa();
+      if (s != SA_OK) return s;
       s = rename(N32, 1, cb, c0, 0, nullptr, nullptr, 0, cur, ctrl->zero);
       if (s != SA_OK) return s;
       s = classify(cur, N / 2 + 1, N32);
@@ -1515,6 +1545,8 @@ struct Build {
     // The unique suffixes' ISA entries are needed only by a later round, the
     // ISA output or the trace; a text resolved in round 0 skips them.
     if (hc.m_next() > 0 || isa_out || want_trace) {
+      s = clear_isa();
+      if (s != SA_OK) return s;
       need_filtered = !isa_out && !opt.trace_isa && !device_rounds_wanted() && N >= NEED_MIN_N &&
                       hc.m_next() <= N / 4;
       if (need_filtered) {

@@ -4,6 +4,11 @@
 // the initial triples (Section 2.1, Algorithm 1): the initial names are
 // built from as many dense codes as fit one 64-bit key.
 //
+// The block that finishes last turns the counts into the dense codes on the
+// device and writes the counts to the host's pinned buffer, so that neither
+// an upload of the codes nor a copy kernel of its own stands on a small
+// text's critical path.
+//
 // Bound: HBM read of n bytes; 16-byte vector loads, per-warp privatised
 // shared-memory counters, one global atomic per bin and block.
 #include "launch.h"
@@ -14,7 +19,10 @@ constexpr int HIST_BLOCK = 512;
 constexpr int HIST_COPIES = HIST_BLOCK / 32;  // one private histogram per warp
 
 __global__ void __launch_bounds__(HIST_BLOCK)
-k_byte_histogram(const uint8_t *__restrict__ text, uint64_t n, uint32_t *__restrict__ hist) {
+k_byte_histogram(AlphabetArgs a) {
+  const uint8_t *__restrict__ text = a.text;
+  const uint64_t n = a.n;
+  uint32_t *hist = a.hist;
   __shared__ uint32_t s_hist[HIST_COPIES][RADIX];
   for (int x = threadIdx.x; x < HIST_COPIES * RADIX; x += HIST_BLOCK) (&s_hist[0][0])[x] = 0;
   __syncthreads();
@@ -46,15 +54,32 @@ k_byte_histogram(const uint8_t *__restrict__ text, uint64_t n, uint32_t *__restr
     for (int c = 0; c < HIST_COPIES; ++c) s += s_hist[c][d];
     if (s) atomicAdd(&hist[d], s);
   }
+  __shared__ uint32_t s_last, s_tmp[HIST_COPIES + 1];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(a.done, 1u) + 1u == gridDim.x ? 1u : 0u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const uint32_t d = threadIdx.x;
+  const uint32_t c = d < RADIX ? load_volatile_u32(hist + d) : 0u;
+  uint32_t sigma;
+  const uint32_t code = block_exclusive<HIST_BLOCK>(c ? 1u : 0u, OpAdd(), 0u, s_tmp, sigma);
+  if (d < RADIX) {
+    a.code[d] = (uint8_t)code;
+    if (a.host) a.host[d] = c;
+  }
+  if (d < 2 && a.seg_off) a.seg_off[d] = d ? (uint32_t)n : 0u;
 }
 
-cudaError_t launch_byte_histogram(const uint8_t *text, uint64_t n, uint32_t *hist, int num_sms,
-                                  cudaStream_t stream) {
-  if (n == 0) return cudaSuccess;
-  uint64_t want = (n / 16 + HIST_BLOCK - 1) / HIST_BLOCK;
+cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream) {
+  if (a.n == 0) return cudaSuccess;
+  uint64_t want = (a.n / 16 + HIST_BLOCK - 1) / HIST_BLOCK;
   uint64_t cap = (uint64_t)num_sms * 4;
   unsigned grid = (unsigned)(want < 1 ? 1 : (want > cap ? cap : want));
-  k_byte_histogram<<<grid, HIST_BLOCK, 0, stream>>>(text, n, hist);
+  k_byte_histogram<<<grid, HIST_BLOCK, 0, stream>>>(a);
   return cudaGetLastError();
 }
 

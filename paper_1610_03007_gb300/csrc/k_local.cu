@@ -151,9 +151,8 @@ __device__ __forceinline__ uint32_t next_head(const uint32_t *ballots, uint32_t 
 
 }  // namespace
 
-__global__ void __launch_bounds__(LC_BLOCK, 2) k_local(LocalArgs a) {
-  extern __shared__ __align__(128) uint8_t smem_raw[];
-  LcSmem &S = *reinterpret_cast<LcSmem *>(smem_raw);
+// One tile. Every thread of the block calls it; all returns are uniform.
+__device__ __forceinline__ void local_tile(LcSmem &S, const LocalArgs &a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t *__restrict__ K = a.plan->kfinal;
   const uint32_t *__restrict__ V = a.plan->vfinal;
@@ -516,6 +515,24 @@ __global__ void __launch_bounds__(LC_BLOCK, 2) k_local(LocalArgs a) {
     a.act_out[S.surv_base + i] = ((uint64_t)(S.grp_base + o) << 32) | v;
     a.upd[S.upd_base + i] = ((uint64_t)names[o] << 32) | v;
   }
+}
+
+__global__ void __launch_bounds__(LC_BLOCK, 2) k_local(LocalArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  LcSmem &S = *reinterpret_cast<LcSmem *>(smem_raw);
+  local_tile(S, a);
+  if (!a.host) return;
+  // The last tile reports the counts and the error word to the host.
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    S.sq = atomicAdd(&a.ctrl->done[1], 1u) + 1u == gridDim.x ? 1u : 0u;
+  }
+  __syncthreads();
+  if (!S.sq) return;
+  __threadfence();
+  if (threadIdx.x < 16)
+    a.host[threadIdx.x] = load_volatile_u32(reinterpret_cast<const uint32_t *>(a.ctrl) + threadIdx.x);
 }
 
 cudaError_t launch_local(const LocalArgs &a, cudaStream_t stream) {

@@ -176,39 +176,6 @@ __global__ void __launch_bounds__(PACK_BLOCK) k_pack(PackArgs a) {
   }
 }
 
-// The digit histograms of a single text's keys from the top digit's alone,
-// when every digit covers g = 8 / b whole characters (b divides 8 and c0 * b
-// is a multiple of 8): digit p of the key at position i is the g-character
-// gram at i + q_p, q_p = (c0 * b - 8 - shift_p) / b, with code 0 past the end
-// of the text. Over i in [0, n) those grams are the grams at [q_p, n + q_p):
-// the top digit's histogram (q = 0, grams at [0, n)) minus the grams at
-// [0, q_p) plus q_p all-padding grams (digit 0). One block; q_p < 64.
-__global__ void __launch_bounds__(RADIX) k_pack_hist_fixup(PackArgs a) {
-  __shared__ uint8_t s_code[RADIX];
-  __shared__ uint32_t s_gram[64];
-  const uint32_t d = threadIdx.x;
-  s_code[d] = a.code[d];
-  const uint32_t P = a.spec.P, g = 8 / a.b;
-  const uint32_t top = a.hist[(MAX_PASSES - 1) * RADIX + d];
-  __syncthreads();
-  // grams at positions 0 .. 63 (all q_p are below c0 <= 64)
-  if (d < 64) {
-    uint32_t v = 0;
-    for (uint32_t c = 0; c < g; ++c) {
-      const uint64_t x = (uint64_t)d + c;
-      v = (v << a.b) | (x < a.N ? s_code[a.text[x]] : 0u);
-    }
-    s_gram[d] = v;
-  }
-  __syncthreads();
-  for (uint32_t p = 0; p < P; ++p) {
-    const uint32_t qp = (a.cb - 8 - a.spec.shift[p]) / a.b;
-    uint32_t below = 0;
-    for (uint32_t x = 0; x < qp; ++x) below += s_gram[x] == d ? 1u : 0u;
-    a.hist[p * RADIX + d] = top - below + (d == 0 ? qp : 0u);
-  }
-}
-
 // The top digit's histogram alone (keys == NULL, top_only): the g-character
 // gram (g = 8 / B) at every position p in [0, n), code 0 past the end, is
 // the top digit of the key of p whatever index holds it, so no key is
@@ -301,11 +268,6 @@ cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream) {
     const uint64_t span = PACK_BLOCK * 8;
     k_pack<8><<<(unsigned)((a.N + span - 1) / span), PACK_BLOCK, 0, stream>>>(a);
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pack_fixup(const PackArgs &a, cudaStream_t stream) {
-  k_pack_hist_fixup<<<1, RADIX, 0, stream>>>(a);
   return cudaGetLastError();
 }
 

@@ -85,10 +85,20 @@ cudaError_t launch_digit_histogram(const uint64_t *keys, uint32_t m, const Digit
 // DNA or bytes: 28 to 30, where the masks measured faster).
 constexpr float MATCH_RANK_MAX_DISTINCT = 24.f;
 
+// GRAMS: the digit histograms of a single text's keys from the top digit's
+// alone (the last row of hist), when every digit covers g = 8 / b whole
+// characters (b divides 8 and c0 * b is a multiple of 8): digit p of the key
+// at position i is the g-character gram at i + q_p, q_p = (c0 * b - 8 -
+// shift_p) / b, with code 0 past the end of the text. Over i in [0, n) those
+// grams are the grams at [q_p, n + q_p): the top digit's histogram (q = 0,
+// grams at [0, n)) minus the grams at [0, q_p) plus q_p all-padding grams
+// (digit 0); q_p < 64.
+template <bool GRAMS>
 __global__ void __launch_bounds__(RADIX)
 k_sort_plan(const uint32_t *__restrict__ hist, uint32_t *__restrict__ digit_base, DigitSpec spec,
             uint32_t m, uint64_t *ka, uint64_t *kb, uint32_t *va, uint32_t *vb,
-            SortPlan *plan, Ctrl *ctrl, const RoundState *rs, uint32_t keep) {
+            SortPlan *plan, Ctrl *ctrl, const RoundState *rs, uint32_t keep,
+            PackArgs grams) {
   __shared__ uint32_t s_tmp[RADIX / 32 + 1];
   if (rs) {  // device-driven rounds
     if (!rs->live) return;
@@ -100,8 +110,28 @@ k_sort_plan(const uint32_t *__restrict__ hist, uint32_t *__restrict__ digit_base
   __shared__ uint32_t s_match;
   const uint32_t d = threadIdx.x;
   if (d == 0) s_match = 0u;
+  __shared__ uint32_t s_gram[64];
+  uint32_t top = 0;
+  if constexpr (GRAMS) {
+    top = hist[(MAX_PASSES - 1) * RADIX + d];
+    if (d < 64) {  // the grams at positions 0 .. 63
+      uint32_t v = 0;
+      for (uint32_t x = d; x < d + 8 / grams.b; ++x)
+        v = (v << grams.b) | (x < grams.N ? grams.code[grams.text[x]] : 0u);
+      s_gram[d] = v;
+    }
+    __syncthreads();
+  }
   for (uint32_t p = 0; p < spec.P; ++p) {
-    const uint32_t c = hist[p * RADIX + d];
+    uint32_t c;
+    if constexpr (GRAMS) {
+      const uint32_t q = (grams.cb - 8 - spec.shift[p]) / grams.b;
+      uint32_t below = 0;
+      for (uint32_t x = 0; x < q; ++x) below += s_gram[x] == d ? 1u : 0u;
+      c = top - below + (d == 0 ? q : 0u);
+    } else {
+      c = hist[p * RADIX + d];
+    }
     uint32_t total;
     const uint32_t excl = block_exclusive<RADIX>(c, OpAdd(), 0u, s_tmp, total);
     digit_base[p * RADIX + d] = excl;
@@ -160,9 +190,13 @@ k_sort_plan(const uint32_t *__restrict__ hist, uint32_t *__restrict__ digit_base
 cudaError_t launch_sort_plan(const uint32_t *hist, uint32_t *digit_base, const DigitSpec &spec,
                              uint32_t m, uint64_t *ka, uint64_t *kb, uint32_t *va,
                              uint32_t *vb, SortPlan *plan, Ctrl *ctrl, cudaStream_t stream,
-                             const RoundState *rs, uint32_t keep) {
-  k_sort_plan<<<1, RADIX, 0, stream>>>(hist, digit_base, spec, m, ka, kb, va, vb, plan, ctrl, rs,
-                                       keep);
+                             const RoundState *rs, uint32_t keep, const PackArgs *grams) {
+  if (grams)
+    k_sort_plan<true><<<1, RADIX, 0, stream>>>(hist, digit_base, spec, m, ka, kb, va, vb, plan,
+                                               ctrl, rs, keep, *grams);
+  else
+    k_sort_plan<false><<<1, RADIX, 0, stream>>>(hist, digit_base, spec, m, ka, kb, va, vb, plan,
+                                                ctrl, rs, keep, PackArgs{});
   return cudaGetLastError();
 }
 

@@ -36,10 +36,16 @@ cudaError_t launch_copy_words(uint32_t *dst, const uint32_t *src, uint64_t words
 cudaError_t launch_copy_bytes(uint8_t *dst, const uint8_t *src, uint64_t n, cudaStream_t stream);
 
 // ---- step A0: alphabet (k_alphabet.cu) ----------------------------------
-// hist[256] += occurrences of each byte value in text[0, n). hist must be
-// zeroed by the caller.
-cudaError_t launch_byte_histogram(const uint8_t *text, uint64_t n, uint32_t *hist,
-                                  int num_sms, cudaStream_t stream);
+struct AlphabetArgs {
+  const uint8_t *text;
+  uint64_t n;
+  uint32_t *hist;     // 256 counts (zeroed by the caller), += the text's
+  uint32_t *done;     // blocks finished (zeroed by the caller)
+  uint8_t *code;      // out: dense order-preserving code of each byte value
+  uint32_t *seg_off;  // out, for one text: {0, n} (NULL otherwise)
+  uint32_t *host;     // out: the counts in pinned host memory, or NULL
+};
+cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream);
 
 // ---- step A1: initial keys (k_pack.cu) ----------------------------------
 struct PackArgs {
@@ -57,7 +63,7 @@ struct PackArgs {
   uint32_t *hist;          // out: += their histograms (P * 256, zeroed by the caller)
   // 1: one text whose digits hold whole characters (b divides 8, cb a
   // multiple of 8): only the top digit is counted per key and the other
-  // histograms are derived from it (launch_pack_fixup).
+  // histograms are derived from it (launch_sort_plan).
   uint32_t top_only;
 };
 // keys == NULL (top_only only): only the top digit's histogram (the first
@@ -65,7 +71,6 @@ struct PackArgs {
 // top_only the counts go to the last of the MAX_PASSES rows, from which
 // launch_pack_fixup derives the rows of the digits in spec.
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream);
-cudaError_t launch_pack_fixup(const PackArgs &a, cudaStream_t stream);
 
 // ---- step A2: radix sort (k_sort.cu) ------------------------------------
 // hist[P*256] += digit counts of keys[0, m) for the digits in spec.
@@ -78,10 +83,13 @@ cudaError_t launch_digit_histogram(const uint64_t *keys, uint32_t m, const Digit
 // keep: bit p keeps pass p even if its digit is constant (the pass that
 // reads the text, PassArgs.text; every pass, so that the host knows which
 // buffer the result is in).
+// grams: the histograms of a text's keys are derived from the last row of
+// hist first (PackArgs.top_only).
 cudaError_t launch_sort_plan(const uint32_t *hist, uint32_t *digit_base, const DigitSpec &spec,
                              uint32_t m, uint64_t *ka, uint64_t *kb, uint32_t *va,
                              uint32_t *vb, SortPlan *plan, Ctrl *ctrl, cudaStream_t stream,
-                             const RoundState *rs = nullptr, uint32_t keep = 0);
+                             const RoundState *rs = nullptr, uint32_t keep = 0,
+                             const PackArgs *grams = nullptr);
 // One stable one-sweep pass over digit p of the plan.
 struct PassArgs {
   const SortPlan *plan;
@@ -184,6 +192,7 @@ struct LocalArgs {
   uint32_t *lg, *loff, *lbase, *lold;
   uint32_t max_large, max_groups;
   Ctrl *ctrl;               // rc.m_s / rc.g_s / rc.upd reserve the outputs
+  uint32_t *host;           // the last tile copies the head of ctrl here (pinned; or NULL)
 };
 cudaError_t launch_local(const LocalArgs &a, cudaStream_t stream);
 struct GatherBigArgs {
