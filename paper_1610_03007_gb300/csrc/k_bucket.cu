@@ -71,6 +71,7 @@ __device__ __forceinline__ bool translate(const BucketArgs &a, uint64_t &e) {
 }  // namespace
 
 __global__ void __launch_bounds__(256, 4) k_bucket_count(BucketArgs a) {
+  if (a.only_if && *a.only_if == 0u) return;
   __shared__ uint32_t bins[RADIX];
   const uint32_t t = threadIdx.x;
   bins[t] = 0u;
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(256, 4) k_bucket_count(BucketArgs a) {
 
 // One block: counts[b][k] -> start of block b's run in bucket k.
 __global__ void __launch_bounds__(256) k_bucket_offsets(BucketArgs a, uint32_t blocks) {
+  if (a.only_if && *a.only_if == 0u) return;
   __shared__ uint32_t wtot[8];
   const uint32_t k = threadIdx.x, lane = k & 31, warp = k >> 5;
   uint32_t total = 0;
@@ -126,6 +128,7 @@ __global__ void __launch_bounds__(256) k_bucket_offsets(BucketArgs a, uint32_t b
 // grouped by bucket, then write it out so that consecutive threads store
 // consecutive slots of each bucket run.
 __global__ void __launch_bounds__(256, 4) k_bucket_scatter(BucketArgs a) {
+  if (a.only_if && *a.only_if == 0u) return;
   __shared__ uint64_t stage[BK_CHUNK];
   __shared__ uint32_t run[RADIX], cnt[RADIX], at0[RADIX], lofs[RADIX];
   __shared__ uint32_t wtot[8];

@@ -435,6 +435,7 @@ struct BucketArgs {
   const uint64_t *in;     // entries (x << 32) | i'
   const uint32_t *lo;     // device word: first entry (NULL: 0)
   const uint32_t *count;  // device word: number of entries
+  const uint32_t *only_if;  // device word: nothing is done when it is 0 (NULL: always)
   uint32_t max_count;     // capacity of `in` past *lo and of `out`
   uint32_t shift;         // bucket of an entry: min(i' >> shift, 255)
   uint32_t blocks;        // partition blocks (<= BUCKET_BLOCKS_MAX)
