@@ -662,6 +662,7 @@ struct Build {
     ca.lold = lold;
     ca.tfirst = tfirst;
     ca.nominal = nominal;
+    ca.small = REFINE_SHAPE[shape].small;
     ca.max_groups = L.max_groups;
     ca.max_tiles = L.max_tiles;
     ca.ctrl = ctrl;
@@ -978,6 +979,7 @@ struct Build {
     ca.lold = lold;
     ca.tfirst = tfirst;
     ca.nominal = nominal;
+    ca.small = REFINE_SHAPE[shape].small;
     ca.max_groups = L.max_groups;
     ca.max_tiles = L.max_tiles;
     ca.ctrl = ctrl;
@@ -1450,7 +1452,7 @@ struct Build {
                       items_ok(opt.sort_items), items_ok(tuned.sort_items));
     shape = pick(opt.refine_shape, tuned.refine_shape, 1, shape_ok(opt.refine_shape),
                  shape_ok(tuned.refine_shape)) - 1;
-    nominal = REFINE_SHAPE[shape].cap / 2;
+    nominal = REFINE_SHAPE[shape].window();
     bucket_min = pick(opt.bucket_min, tuned.bucket_min, BUCKET_MIN, true, true);
     const uint32_t h0 = pick(opt.h0_chars, tuned.h0_chars, 0, true, true);
     uint32_t c0 = (64 - segbits) / b;

@@ -6,8 +6,8 @@
 // crosses group boundaries. So the sort of a round is a segmented sort, and
 // a group that fits one tile can be refined entirely inside one block:
 //
-//   k_refine (one tile = whole groups whose starts fall in a 2048-item
-//   window, at most 4096 items): load the tile's (g, i') from the active
+//   k_refine (one tile = whole groups whose starts fall in the tile's
+//   window): load the tile's (g, i') from the active
 //   list, gather the partner names r2 = ISA[i' + h] + 1 (Algorithm 4), sort
 //   by (local group, r2) with a radix sort in shared memory, then rename
 //   (CmpName + max PrefixSum inside the tile; NameDiscarding's
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) k_classify(ClassifyArgs a) {
             name = head;
           a.gname[x] = name;
         }
-        if (size > a.nominal) {
+        if (size > a.small) {
           if (x < gs) name = a.gname[x];
           const unsigned long long old =
               atomicAdd(&a.ctrl->rc.large, (1ull << 32) | (unsigned long long)size);
@@ -250,14 +250,21 @@ cudaError_t launch_wide_finish(const WideArgs &a, cudaStream_t stream) {
 constexpr uint32_t RF_RANK_GMAX = GBSA_RF_RANK_GMAX;
 constexpr uint32_t RF_RANK_AVG = GBSA_RF_RANK_AVG;
 
+constexpr int rf_small(int block, int cap) {
+  for (const RefineShape &s : REFINE_SHAPE)
+    if ((int)s.block == block && (int)s.cap == cap) return (int)s.small;
+  return 0;
+}
+
 template <int BLOCK, int CAP>
 struct RfCfg {
   static constexpr int WARPS = BLOCK / 32;
   static constexpr int ITEMS = CAP / BLOCK;       // slots per thread
-  static constexpr int NOMINAL = CAP / 2;         // tile window and largest small group
-  static constexpr int MAXG = NOMINAL / 2 + 1;    // groups have >= 2 members
+  static constexpr int SMALL = rf_small(BLOCK, CAP);   // largest small group
+  static constexpr int MAXG = (CAP - SMALL) / 2 + 1;   // starts in a window: groups have >= 2 members
   static constexpr int GPT = (MAXG + BLOCK - 1) / BLOCK;  // groups per thread
   static constexpr int DPT = RADIX / BLOCK;       // digits per thread in the digit scan
+  static constexpr int SEGS = CAP / 32;           // rows of 32 items
   static_assert(ITEMS >= 1 && ITEMS <= 16, "slots per thread");
   static_assert(DPT >= 1 && RADIX % BLOCK == 0, "digits per thread");
 };
@@ -274,6 +281,13 @@ struct RfWide {
 template <int CAP>
 struct RfWide<CAP, false> {};
 
+// Per local group (refine_pivot): its first member's partner name and the
+// number of members with a smaller one.
+template <int MAXG>
+struct RfPivot {
+  uint32_t name[MAXG], less[MAXG];
+};
+
 template <int BLOCK, int CAP, bool WIDE>
 struct RfSmem {
   using C = RfCfg<BLOCK, CAP>;
@@ -286,8 +300,15 @@ struct RfSmem {
     // measured fastest (the same shape with 3 KB less shared memory ran the
     // refine about 5% slower on GB300).
     uint32_t spacer[C::WARPS][RADIX];
+    // refine_pivot: the items off their group's pivot, in group order.
+    struct {
+      uint32_t ip[C::WARPS * RADIX / 4], name[C::WARPS * RADIX / 4], lg[C::WARPS * RADIX / 4];
+    } off;
   };
-  uint16_t whist[2][C::WARPS][RADIX];   // per pass (double-buffered): counts, then prefixes
+  union {
+    uint16_t whist[2][C::WARPS][RADIX];  // per pass (double-buffered): counts, then prefixes
+    RfPivot<C::MAXG> pv;
+  };
   uint32_t dstart[RADIX];
   uint32_t gname[C::MAXG];
   uint32_t ghead[C::MAXG];              // head rank (SA interval start) of the local group
@@ -296,6 +317,12 @@ struct RfSmem {
   uint32_t flag, all_small, upd_local, upd_base, surv_base, grp_base;
   uint32_t gmax, gsq;  // largest small group, sum of squared small-group sizes
   unsigned long long orv, orv2;
+  uint32_t pairs;  // comparisons refine_pivot would make
+  // refine_pivot: marks by sorted position (survivor 1, head of a surviving
+  // subgroup 2, changed name 4), their ballots and counts.
+  uint8_t mark[CAP];
+  uint32_t surv[C::SEGS], heads[C::SEGS];
+  unsigned long long seg[C::SEGS + 1];  // then their exclusive sums and the total
 };
 
 // One-barrier exclusive sum over the block: warp scans, warp totals in
@@ -490,6 +517,32 @@ __device__ void rf_tile_sort(RfSmem<BLOCK, CAP, WIDE> &S, uint32_t cnt,
 // sorted order has the SA interval [head + a, head + a + len).
 constexpr uint32_t RF_GROUP_MAX = 4;
 
+// Exclusive sums of v[0, N) by one warp, the total in v[N].
+template <int N>
+__device__ __forceinline__ void rf_scan_segments(unsigned long long *v) {
+  constexpr int PER = N / 32;
+  const int lane = threadIdx.x & 31;
+  unsigned long long c[PER], sum = 0;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    c[i] = v[lane * PER + i];
+    sum += c[i];
+  }
+  unsigned long long incl = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  unsigned long long run = incl - sum;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    v[lane * PER + i] = run;
+    run += c[i];
+  }
+  if (lane == 31) v[N] = incl;
+}
+
 // Exclusive sum over the block of 64-bit values (one barrier), the total in
 // `total`; `tmp` holds 2 * WARPS words and is not rewritten before the
 // next barrier.
@@ -655,6 +708,206 @@ __device__ __forceinline__ void refine_tiny_groups(RfSmem<BLOCK, CAP, false> &S,
   }
 }
 
+// Tiles of larger groups: the members of a group of repeats mostly share
+// their partner name, so instead of sorting the tile, every member is
+// compared with its group's first partner name (the pivot). Members with the
+// pivot's name form one subgroup, in the order of the list; ballots and one
+// scan number the others, which are gathered densely in group order and find
+// their places by comparing with their group's part of that short list, one
+// thread each. Places, subgroup bounds and names follow from the counts, so
+// the outputs need one more scan, of ballots over the sorted positions: no
+// sort, no rank atomics.
+//
+// Returns false, with nothing written, when too many items are off their
+// pivots: the tile is then sorted. All returns are block-uniform.
+//
+// Bound: barriers and shared-memory latency (issue active 46 %, DRAM 10 %).
+// Refine of the 2^26 repeated Zipf text, 256 x 2048 tiles: in-tile radix
+// sort 13.97 ms, this 12.7 (10.7 with the wider window of REFINE_SHAPE).
+// Every item comparing with its group's list in place (a warp waits for its
+// longest list), ranks by match.any: 13.6.
+//
+// Comparisons per item of the tile up to which the lists pay (8, 32, 100,
+// 300: 12.98, 12.83, 12.67, 12.73 ms).
+constexpr uint32_t RF_PIVOT_AVG = 100;
+
+template <int BLOCK, int CAP>
+__device__ __forceinline__ bool refine_pivot(RfSmem<BLOCK, CAP, false> &S, const RefineArgs &a,
+                                             const uint64_t (&ent)[CAP / BLOCK],
+                                             const uint32_t (&r2)[CAP / BLOCK], const uint32_t g0,
+                                             const uint32_t ng, const uint32_t cnt,
+                                             const uint32_t K) {
+  using C = RfCfg<BLOCK, CAP>;
+  constexpr uint32_t OFF_MAX = C::WARPS * RADIX / 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
+  uint32_t *names = reinterpret_cast<uint32_t *>(S.keys);  // new names by sorted position
+  for (uint32_t g = tid; g < ng; g += BLOCK) S.pv.less[g] = 0u;
+#pragma unroll
+  for (int k = 0; k < C::ITEMS; ++k) {
+    const uint32_t q = k * BLOCK + tid;
+    if ((uint32_t)k < K && q < cnt) {
+      const uint32_t lg = (uint32_t)(ent[k] >> 32) - g0;
+      if (q == S.goff[lg]) S.pv.name[lg] = r2[k];
+    }
+  }
+  __syncthreads();
+  // Items off their pivot: bits in list order (S.surv) and their counts.
+  uint32_t offbits = 0;
+#pragma unroll
+  for (int k = 0; k < C::ITEMS; ++k) {
+    const uint32_t q = k * BLOCK + tid;
+    bool off = false;
+    if ((uint32_t)k < K && q < cnt) {
+      const uint32_t lg = (uint32_t)(ent[k] >> 32) - g0, pivot = S.pv.name[lg];
+      off = r2[k] != pivot;
+      if (r2[k] < pivot) atomicAdd(&S.pv.less[lg], 1u);
+    }
+    const uint32_t B = __ballot_sync(0xffffffffu, off);
+    if (lane == 0) {
+      S.surv[k * C::WARPS + warp] = B;
+      S.seg[k * C::WARPS + warp] = __popc(B);
+    }
+    offbits |= (uint32_t)off << k;
+  }
+  __syncthreads();
+  if (warp == 0) rf_scan_segments<C::SEGS>(S.seg);
+  __syncthreads();
+  const uint32_t noff = (uint32_t)S.seg[C::SEGS];
+  if (noff > OFF_MAX) return false;
+  // Items off their pivots before item q of the list (q <= cnt).
+  auto off_before = [&](uint32_t q) -> uint32_t {
+    if (q >= (uint32_t)CAP) return noff;
+    return (uint32_t)S.seg[q >> 5] + __popc(S.surv[q >> 5] & ((1u << (q & 31)) - 1u));
+  };
+  // place: position | mark << 16. An item on its pivot follows the smaller
+  // ones of its group, in list order.
+  uint32_t place[C::ITEMS], pairs = 0;
+#pragma unroll
+  for (int k = 0; k < C::ITEMS; ++k) {
+    place[k] = 0;
+    const uint32_t q = k * BLOCK + tid;
+    if ((uint32_t)k >= K || q >= cnt) continue;
+    const uint32_t lg = (uint32_t)(ent[k] >> 32) - g0;
+    const uint32_t start = S.goff[lg], end = S.goff[lg + 1];
+    const uint32_t o0 = off_before(start), n = off_before(end) - o0;
+    const uint32_t i = (uint32_t)S.seg[q >> 5] + __popc(S.surv[q >> 5] & lt);
+    if ((offbits >> k) & 1u) {
+      S.off.ip[i] = (uint32_t)ent[k];
+      S.off.name[i] = r2[k];
+      S.off.lg[i] = lg;
+      pairs += n;
+      continue;
+    }
+    const uint32_t head = start + S.pv.less[lg], len = end - start - n;
+    const uint32_t pos = head + (q - start) - (i - o0);
+    const uint32_t lo = S.ghead[lg] + (head - start), old = S.gname[lg];
+    const uint32_t name = a.naming != NAMES_RETAIN ? lo : (old - lo < len ? old : lo + len / 2);
+    const uint32_t mark =
+        (len > 1 ? 1u : 0u) | (len > 1 && pos == head ? 2u : 0u) | (name != old ? 4u : 0u);
+    place[k] = pos | (mark << 16);
+    S.vals[pos] = (uint32_t)ent[k];
+    names[pos] = name;
+    S.mark[pos] = (uint8_t)mark;
+  }
+  pairs = __reduce_add_sync(0xffffffffu, pairs);
+  if (lane == 0 && pairs) atomicAdd(&S.pairs, pairs);
+  __syncthreads();
+  if (S.pairs > RF_PIVOT_AVG * cnt) return false;
+  for (uint32_t t = tid; t < noff; t += BLOCK) {
+    const uint32_t r = S.off.name[t], lg = S.off.lg[t], ip = S.off.ip[t];
+    const uint32_t start = S.goff[lg], end = S.goff[lg + 1];
+    const uint32_t o0 = off_before(start), o1 = off_before(end);
+    uint32_t smaller = 0, equal = 0, before = 0;
+    for (uint32_t x = o0; x < o1; ++x) {
+      const uint32_t o = S.off.name[x];
+      smaller += o < r ? 1u : 0u;
+      equal += o == r ? 1u : 0u;
+      before += o == r && x < t ? 1u : 0u;
+    }
+    const uint32_t head =
+        start + smaller + (r > S.pv.name[lg] ? end - start - (o1 - o0) : 0u), pos = head + before;
+    const uint32_t lo = S.ghead[lg] + (head - start), old = S.gname[lg];
+    const uint32_t name =
+        a.naming != NAMES_RETAIN ? lo : (old - lo < equal ? old : lo + equal / 2);
+    const uint32_t mark =
+        (equal > 1 ? 1u : 0u) | (equal > 1 && before == 0 ? 2u : 0u) | (name != old ? 4u : 0u);
+    S.off.ip[t] = pos | (mark << 16);
+    S.vals[pos] = ip;
+    names[pos] = name;
+    S.mark[pos] = (uint8_t)mark;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < C::ITEMS; ++k) {
+    const uint32_t e = k * BLOCK + tid;
+    const uint32_t m = (uint32_t)k < K && e < cnt ? S.mark[e] : 0u;
+    const uint32_t Sv = __ballot_sync(0xffffffffu, m & 1u), H = __ballot_sync(0xffffffffu, m & 2u);
+    const uint32_t Ch = __ballot_sync(0xffffffffu, m & 4u);
+    if (lane == 0) {
+      S.surv[k * C::WARPS + warp] = Sv;
+      S.heads[k * C::WARPS + warp] = H;
+      S.seg[k * C::WARPS + warp] = (unsigned long long)__popc(Sv) |
+                                   ((unsigned long long)__popc(H) << 21) |
+                                   ((unsigned long long)__popc(Ch) << 42);
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {  // the tile's output space
+    rf_scan_segments<C::SEGS>(S.seg);
+    if (lane == 31) {
+      const unsigned long long tot = S.seg[C::SEGS];
+      const uint32_t tot_surv = (uint32_t)(tot & 0x1FFFFFu);
+      const uint32_t tot_grp = (uint32_t)((tot >> 21) & 0x1FFFFFu), tot_chg = (uint32_t)(tot >> 42);
+      const unsigned long long old =
+          tot_surv ? atomicAdd(reinterpret_cast<unsigned long long *>(&a.ctrl->rc.m_s),
+                               ((unsigned long long)tot_grp << 32) | tot_surv)
+                   : 0ull;
+      S.surv_base = (uint32_t)old;
+      S.grp_base = (uint32_t)(old >> 32);
+      S.upd_base = tot_chg ? atomicAdd(&a.ctrl->rc.upd, tot_chg) : 0u;
+    }
+  }
+  __syncthreads();
+  // The heads of surviving subgroups, by the threads that hold them.
+  auto write_head = [&](uint32_t pm, uint32_t lg) {
+    if (!((pm >> 17) & 1u)) return;
+    const uint32_t pos = pm & 0xFFFFu, w = pos >> 5, m = (1u << (pos & 31)) - 1u;
+    const uint32_t g = S.grp_base + (uint32_t)((S.seg[w] >> 21) & 0x1FFFFFu) + __popc(S.heads[w] & m);
+    a.gstart_out[g] = S.surv_base + (uint32_t)(S.seg[w] & 0x1FFFFFu) + __popc(S.surv[w] & m);
+    a.gname_out[g] = names[pos];
+    a.ghead_out[g] = S.ghead[lg] + (pos - S.goff[lg]);
+  };
+#pragma unroll
+  for (int k = 0; k < C::ITEMS; ++k) write_head(place[k], (uint32_t)(ent[k] >> 32) - g0);
+  for (uint32_t t = tid; t < noff; t += BLOCK) write_head(S.off.ip[t], S.off.lg[t]);
+#pragma unroll
+  for (int k = 0; k < C::ITEMS; ++k) {
+    if ((uint32_t)k >= K) continue;  // block-uniform
+    const uint32_t e = k * BLOCK + tid;
+    const uint32_t m = e < cnt ? S.mark[e] : 0u;
+    const uint32_t Ch = __ballot_sync(0xffffffffu, m & 4u);
+    if (e >= cnt) continue;
+    const uint32_t w = k * C::WARPS + warp, ip = S.vals[e], name = names[e];
+    if (name >= a.N || ip >= a.isa_len) {  // never taken unless a logic error
+      raise_error(a.ctrl, ERR_INTERNAL, 24);
+      continue;
+    }
+    const unsigned long long pre = S.seg[w];
+    if (m & 4u)
+      a.upd[S.upd_base + (uint32_t)(pre >> 42) + __popc(Ch & lt)] = ((uint64_t)name << 32) | ip;
+    if (m & 1u) {
+      const uint32_t g = S.grp_base + (uint32_t)((pre >> 21) & 0x1FFFFFu) +
+                         __popc(S.heads[w] & (lt | (1u << lane))) - 1u;
+      a.act_out[S.surv_base + (uint32_t)(pre & 0x1FFFFFu) + __popc(S.surv[w] & lt)] =
+          ((uint64_t)g << 32) | ip;
+    } else {
+      a.sa[name] = local_index(ip, a.seg_off, a.S);
+    }
+  }
+  return true;
+}
+
 // One refine tile (whole groups whose starts fall in the tile's window).
 // Every thread of the block calls it; all returns are block-uniform.
 template <int BLOCK, int CAP, bool WIDE>
@@ -668,6 +921,7 @@ __device__ __forceinline__ void refine_tile(RfSmem<BLOCK, CAP, WIDE> &S, const R
     S.upd_local = 0u;
     S.gmax = 0u;
     S.gsq = 0u;
+    S.pairs = 0u;
     S.flag = has_error(a.ctrl) ? 1u : 0u;
   }
   __syncthreads();
@@ -695,7 +949,7 @@ __device__ __forceinline__ void refine_tile(RfSmem<BLOCK, CAP, WIDE> &S, const R
       S.gname[lg] = __ldg(a.gname + g);
       S.ghead[lg] = __ldg(a.ghead + g);
       const uint32_t size = e - s;
-      if (size <= (uint32_t)C::NOMINAL)
+      if (size <= (uint32_t)C::SMALL)
         sz[r] = size;
       else
         mybig = 1;
@@ -779,6 +1033,11 @@ __device__ __forceinline__ void refine_tile(RfSmem<BLOCK, CAP, WIDE> &S, const R
       r2v[k] = __ldg(a.isa + at) + 1u;
     }
   }
+  // Tiles of small groups only are ordered by counting (below).
+  const bool by_rank = S.gmax <= RF_RANK_GMAX && S.gsq <= RF_RANK_AVG * cnt;
+  if constexpr (!WIDE) {
+    if (!by_rank && refine_pivot<BLOCK, CAP>(S, a, ent, r2v, g0, ng, cnt, K)) return;
+  }
   // a = 3, 4 (Prefix Quadrupling): the names of i' + 2h and i' + 3h as well,
   // 0 once an earlier one is the end sentinel (ties on a non-zero name
   // imply the later offsets stay inside the text; the rest never decide).
@@ -828,7 +1087,7 @@ __device__ __forceinline__ void refine_tile(RfSmem<BLOCK, CAP, WIDE> &S, const R
   // list, which is the stable sort's order, at about (sum of squared group
   // sizes) / items comparisons per item instead of the radix passes.
   if constexpr (!WIDE) {
-    if (S.gmax <= RF_RANK_GMAX && S.gsq <= RF_RANK_AVG * cnt) {
+    if (by_rank) {
       uint32_t dst[C::ITEMS];
 #pragma unroll
       for (int k = 0; k < C::ITEMS; ++k) {

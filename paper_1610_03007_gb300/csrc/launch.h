@@ -242,16 +242,23 @@ cudaError_t launch_need_collect(const CollectArgs &a, int num_sms, cudaStream_t 
 // Groups of up to REFINE_SMALL_MAX members are refined inside one tile
 // (gather, shared-memory sort, rename, compaction); larger ones go through
 // the global radix sort and k_rename.
-// Tile shapes of the refine (threads per block, items one tile can hold).
-// Tile t owns the groups whose starts fall in [t, t+1) * cap/2 of the
-// active list, so groups of up to cap/2 members are "small".
+// Tile shapes of the refine: threads per block, items one tile can hold, and
+// the largest small group. Tile t owns the groups whose starts fall in
+// [t, t+1) * (cap - small) of the active list, so a tile's groups always fit.
+// The first two shapes' wider windows spread a tile's fixed work over more
+// items; groups above the limit cost more in the global sort. Refine of the
+// 2^28 repeated Zipf text (groups of about 250) with 256 x 2048 tiles and
+// groups of up to 1024, 768, 640, 512: 51.3, 46.4, 44.8, 43.6 ms; of 2^28
+// Markov DNA (pairs) with 128 x 1024 and up to 512, 384, 256: 3.78, 3.39,
+// 4.00 ms.
 struct RefineShape {
-  uint32_t block, cap;
+  uint32_t block, cap, small;
+  constexpr uint32_t window() const { return cap - small; }
 };
 constexpr int REFINE_SHAPES = 4;
-constexpr RefineShape REFINE_SHAPE[REFINE_SHAPES] = {{128, 1024}, {256, 2048}, {256, 4096},
-                                                     {256, 1024}};
-constexpr uint32_t REFINE_MIN_NOMINAL = 512;  // smallest cap/2 (buffer sizing)
+constexpr RefineShape REFINE_SHAPE[REFINE_SHAPES] = {
+    {128, 1024, 384}, {256, 2048, 512}, {256, 4096, 2048}, {256, 1024, 512}};
+constexpr uint32_t REFINE_MIN_NOMINAL = 256;  // least window and least small (buffer sizing)
 
 // Names of groups. A name may be any rank inside the group's SA interval:
 // intervals are disjoint and ordered, so such names respect the order of
@@ -273,7 +280,7 @@ struct ClassifyArgs {
   uint32_t *lg, *loff, *lbase, *lold;  // large groups: index, start in the large
                                        // list, head - start, name
   uint32_t *tfirst;         // first group of each refine tile (tiles + 1 entries)
-  uint32_t nominal;         // refine tile window (cap / 2); also the largest small group
+  uint32_t nominal, small;  // refine tile window; the largest small group
   uint32_t max_groups;      // upper bound of G (buffer capacity)
   uint32_t max_tiles;       // upper bound of tiles (buffer capacity - 1)
   Ctrl *ctrl;               // reads rc.m_s + rc.m_l, rc.g_s + rc.g_l; adds to rc.large
