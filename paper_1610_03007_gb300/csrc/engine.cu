@@ -242,9 +242,16 @@ struct PinnedStage {
 };
 
 // Costs of round 0's steps over all items in units of one radix pass, and
-// a pass's time: a fixed part and 7 ps per item (choose_split).
-constexpr double LOCAL_COST = 1.9, RENAME_COST = 1.5;
+// a pass's time: a fixed part and 7 ps per item (choose_split). The tile
+// pass costs LOCAL_COST, more for larger buckets (per doubling) and, in
+// buckets of more than one item, for skewed digits (by the deviation of
+// -log2 p over 8 bits). Measured against the model at 2^28: DNA after 3, 4, 5
+// passes 1.92, 1.55, 1.40 (1.93, 1.45, 1.45), Markov DNA after 4 and 5 3.4
+// and 2.7 (3.3, 2.1), Zipf bytes at 2^25 after 4 and 5 3.1 and 2.3 (3.2, 2.1).
+constexpr double LOCAL_COST = 1.45, LOCAL_SIZE_COST = 0.06, LOCAL_SKEW_COST = 0.8;
+constexpr double RENAME_COST = 1.5;
 constexpr double PASS_FIXED_US = 9.0, PASS_ITEM_US = 7e-6;
+constexpr uint64_t LOCAL_REPORT_MAX = 1ull << 22;
 // log2 of the bucket size that a tile takes about half of the time: buckets
 // of up to 512 items always fit, of 3072 and more never.
 constexpr double LOCAL_LARGE_LOG2 = 10.3;
@@ -310,16 +317,33 @@ struct PrefixModel {
     return m;
   }
 
-  // Share of a text of 2^log_len characters whose `chars`-character prefix
-  // occurs more than 2^log_large times.
-  double large_share(double chars, double log_len, double log_large) const {
-    if (chars <= 0) return log_len > log_large ? 1.0 : 0.0;
-    double mu = mean * chars / g, v = var * chars / g, top = least * chars / g;
+  // Mean and variance of -log2 p of a `chars`-character prefix, and its least.
+  void prefix(double chars, double &mu, double &v, double &top) const {
+    mu = mean * chars / g, v = var * chars / g, top = least * chars / g;
     if (chars > g) {
       mu = mean + (chars - g) * mean1;
       v = var + (chars - g) * var1;
       top = least + (chars - g) * least1;
     }
+  }
+
+  // Cost of the tile pass over buckets of `chars`-character prefixes of a text
+  // of 2^log_len characters; digit_chars characters to 8 bits.
+  double local_cost(double chars, double log_len, double digit_chars) const {
+    double mu, v, top;
+    prefix(chars, mu, v, top);
+    const double size = log_len - mu, sd = std::sqrt(std::max(v, 0.05));
+    const double shared = 0.5 * std::erfc(-size / (sd * std::sqrt(2.0)));
+    return LOCAL_COST + LOCAL_SIZE_COST * std::max(0.0, size + 4.0) +
+           LOCAL_SKEW_COST * std::sqrt(var1 * digit_chars) * shared;
+  }
+
+  // Share of a text of 2^log_len characters whose `chars`-character prefix
+  // occurs more than 2^log_large times.
+  double large_share(double chars, double log_len, double log_large) const {
+    if (chars <= 0) return log_len > log_large ? 1.0 : 0.0;
+    double mu, v, top;
+    prefix(chars, mu, v, top);
     if (log_len - top < log_large - 1.0) return 0.0;
     const double z = (log_large - (log_len - mu)) / std::sqrt(2.0 * std::max(v, 0.05));
     return 0.5 * std::erfc(z);
@@ -1216,7 +1240,9 @@ struct Build {
     la.max_large = L.max_large;
     la.max_groups = L.max_groups;
     la.ctrl = ctrl;
-    if (stage_readbacks) la.host = reinterpret_cast<uint32_t *>(stage.p);
+    // The last tile's report saves a copy kernel (about 5 us); a tile's share
+    // of it, a fence and an atomic at its end, costs 6 % of long ones.
+    if (stage_readbacks && N <= LOCAL_REPORT_MAX) la.host = reinterpret_cast<uint32_t *>(stage.p);
     sa_status s = launch(SA_K_RENAME, 0, 0, [&] { return launch_local(la, st); });
     if (s != SA_OK) return s;
     if (la.host) {
@@ -1341,8 +1367,8 @@ struct Build {
 
   // Digits of the top that the radix sort of round 0 takes before the
   // buckets are sorted tile by tile, or 0 for all digits: the cheapest by
-  // the model of the prefixes, in units of one pass over all items. A tile
-  // pass costs LOCAL_COST, the rename that it replaces RENAME_COST; items
+  // the model of the prefixes, in units of one pass over all items. The
+  // rename that the tile pass replaces costs RENAME_COST; items
   // in buckets too large for a tile are gathered, sorted by the remaining
   // digits and the bucket ordinal, and renamed.
   uint32_t choose_split(const PrefixModel &model, uint32_t b, uint32_t segbits,
@@ -1354,19 +1380,25 @@ struct Build {
     double best = P + RENAME_COST;
     uint32_t split = 0;
     // Characters by the logarithm of their text's length.
-    double mass[33] = {};
+    double mass[33] = {}, count[33] = {}, log_len[33] = {};
     for (uint32_t k = 0; k < S; ++k) {
       const uint64_t len = off[k + 1] - off[k];
-      if (len) mass[bits_for(len) - 1] += (double)len / (double)N;
+      if (!len) continue;
+      mass[bits_for(len) - 1] += (double)len / (double)N;
+      count[bits_for(len) - 1] += 1.0;
     }
+    for (int l = 0; l < 33; ++l)
+      if (count[l] > 0.0) log_len[l] = std::log2(mass[l] * (double)N / count[l]);
     for (uint32_t p = 1; p * RADIX_BITS < bits0; ++p) {
       const uint32_t T = p * RADIX_BITS;
       const double chars = T > segbits ? (double)(T - segbits) / b : 0.0;
-      double big = 0.0;
+      double big = 0.0, cost = p;
       for (int l = 0; l < 33; ++l)
-        if (mass[l] > 0.0) big += mass[l] * model.large_share(chars, l + 0.5, LOCAL_LARGE_LOG2);
+        if (mass[l] > 0.0) {
+          big += mass[l] * model.large_share(chars, log_len[l], LOCAL_LARGE_LOG2);
+          cost += mass[l] * model.local_cost(chars, log_len[l], 8.0 / b);
+        }
       const uint32_t R = bits0 - T;
-      double cost = p + LOCAL_COST;
       if (big > 0.0) {  // its share of a pass, each with the fixed part of one
         const double rest = (R + bits_for((uint64_t)(big * N / 4096.0)) + 7) / 8;
         const double share = (big * N * PASS_ITEM_US + PASS_FIXED_US) / (N * PASS_ITEM_US + PASS_FIXED_US);
