@@ -145,6 +145,14 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
+// Sets a flag in pinned host memory after everything the block's threads
+// wrote there. Every thread of the block calls it.
+__device__ __forceinline__ void report_to_host(uint32_t *flag) {
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) *reinterpret_cast<volatile uint32_t *>(flag) = 1u;
+}
+
 // ---- TMA bulk copies (global -> shared) behind an mbarrier -----------------
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {

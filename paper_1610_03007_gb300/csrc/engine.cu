@@ -29,6 +29,7 @@
 //   u32[N/2+1], large-group lists, the refine tile map, look-back status,
 //   control block, plan, histograms: about 67 bytes per character.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -542,6 +543,30 @@ struct Build {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) memcpy(host, stage.p, bytes);
     return e;
+  }
+
+  // Reports: words that a kernel's last block writes into the stage, then a
+  // flag of its own (in its own cache line), cleared here before the launch.
+  uint32_t *stage_words() { return reinterpret_cast<uint32_t *>(stage.p); }
+  uint32_t *report_flag(int k) {
+    uint32_t *f = stage_words() + 2 * RADIX + 32 * k;
+    __atomic_store_n(f, 0u, __ATOMIC_RELAXED);
+    return f;
+  }
+
+  // Waits for a report: polls its flag for a while (a stream synchronisation
+  // returns about 4 us after the flag is set), then synchronises the stream.
+  // A kernel that fails sets no flag, and the synchronisation returns its
+  // error. With per-launch events the stream is always synchronised.
+  cudaError_t wait_report(const uint32_t *flag) {
+    if (!prof) {
+      const auto t0 = std::chrono::steady_clock::now();
+      do {
+        for (int i = 0; i < 64; ++i)
+          if (__atomic_load_n(flag, __ATOMIC_ACQUIRE)) return cudaSuccess;
+      } while (std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(300));
+    }
+    return cudaStreamSynchronize(st);
   }
 
   sa_status read_ctrl(HostCtrl &hc) {
@@ -1242,12 +1267,15 @@ struct Build {
     la.ctrl = ctrl;
     // The last tile's report saves a copy kernel (about 5 us); a tile's share
     // of it, a fence and an atomic at its end, costs 6 % of long ones.
-    if (stage_readbacks && N <= LOCAL_REPORT_MAX) la.host = reinterpret_cast<uint32_t *>(stage.p);
+    if (stage_readbacks && N <= LOCAL_REPORT_MAX) {
+      la.host = stage_words() + RADIX;
+      la.host_flag = report_flag(1);
+    }
     sa_status s = launch(SA_K_RENAME, 0, 0, [&] { return launch_local(la, st); });
     if (s != SA_OK) return s;
     if (la.host) {
-      CK(cudaStreamSynchronize(st));
-      memcpy(&hc, stage.p, sizeof(hc));
+      CK(wait_report(la.host_flag));
+      memcpy(&hc, la.host, sizeof(hc));
       s = ctrl_status(hc);
     } else {
       s = read_ctrl(hc);
@@ -1446,14 +1474,17 @@ struct Build {
     aa.done = &ctrl->done[0];
     aa.code = code;
     aa.seg_off = S == 1 ? segoff : nullptr;
-    aa.host = stage_readbacks ? reinterpret_cast<uint32_t *>(stage.p) : nullptr;
+    if (stage_readbacks) {
+      aa.host = stage_words();
+      aa.host_flag = report_flag(0);
+    }
     sa_status s =
         launch(SA_K_BYTE_HIST, 0, N, [&] { return launch_byte_histogram(aa, sm_count(), st); });
     if (s != SA_OK) return s;
     uint32_t hh[RADIX];
     if (aa.host) {
-      CK(cudaStreamSynchronize(st));
-      memcpy(hh, stage.p, sizeof(hh));
+      CK(wait_report(aa.host_flag));
+      memcpy(hh, aa.host, sizeof(hh));
     } else {
       CK(fetch(hh, bytehist, sizeof(hh)));
     }

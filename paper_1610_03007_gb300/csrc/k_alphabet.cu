@@ -72,6 +72,7 @@ k_byte_histogram(AlphabetArgs a) {
     if (a.host) a.host[d] = c;
   }
   if (d < 2 && a.seg_off) a.seg_off[d] = d ? (uint32_t)n : 0u;
+  if (a.host) report_to_host(a.host_flag);
 }
 
 cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream) {

@@ -54,8 +54,10 @@ constexpr int LC_W = LOCAL_TILE;
 constexpr int LC_WARPS = LC_BLOCK / 32;
 constexpr int LC_SEGS = LC_ITEMS * LC_WARPS;  // (row, warp) segments of 32 items
 // Bins of at least LC_RUN_MIN items are spread again or found to be runs, in
-// tiles that would make more than LC_AVG comparisons per item.
-constexpr uint32_t LC_RUN_MIN = 16, LC_AVG = 6;
+// tiles that would make more than LC_AVG comparisons per item. (16 and 6, 16
+// and 24, 64 and 48 against these: 8 M characters of prose 0.50, 0.48, 0.49
+// and 0.46 ms, 2^25 Zipf bytes 0.575, 0.551, 0.559 and 0.551 ms.)
+constexpr uint32_t LC_RUN_MIN = 32, LC_AVG = 12;
 constexpr uint32_t LC_NO_ITEM = 0xFFFFFFFFu;
 constexpr uint32_t LC_MIXED = 0x80000000u;  // bin flag: not one run of equal keys
 static_assert(LC_W % LC_BLOCK == 0 && LC_CAP > LC_W && LC_CAP < 0x8000, "window of whole rows");
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(LC_BLOCK, 2) k_local(LocalArgs a) {
   // The last tile reports the counts and the error word to the host.
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
+    __threadfence_system();  // the host may act on the report before the kernel ends
     S.sq = atomicAdd(&a.ctrl->done[1], 1u) + 1u == gridDim.x ? 1u : 0u;
   }
   __syncthreads();
@@ -533,6 +535,7 @@ __global__ void __launch_bounds__(LC_BLOCK, 2) k_local(LocalArgs a) {
   __threadfence();
   if (threadIdx.x < 16)
     a.host[threadIdx.x] = load_volatile_u32(reinterpret_cast<const uint32_t *>(a.ctrl) + threadIdx.x);
+  report_to_host(a.host_flag);
 }
 
 cudaError_t launch_local(const LocalArgs &a, cudaStream_t stream) {

@@ -44,6 +44,7 @@ struct AlphabetArgs {
   uint8_t *code;      // out: dense order-preserving code of each byte value
   uint32_t *seg_off;  // out, for one text: {0, n} (NULL otherwise)
   uint32_t *host;     // out: the counts in pinned host memory, or NULL
+  uint32_t *host_flag;  // set to 1 after them
 };
 cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream);
 
@@ -193,6 +194,7 @@ struct LocalArgs {
   uint32_t max_large, max_groups;
   Ctrl *ctrl;               // rc.m_s / rc.g_s / rc.upd reserve the outputs
   uint32_t *host;           // the last tile copies the head of ctrl here (pinned; or NULL)
+  uint32_t *host_flag;      // and sets this to 1
 };
 cudaError_t launch_local(const LocalArgs &a, cudaStream_t stream);
 struct GatherBigArgs {
