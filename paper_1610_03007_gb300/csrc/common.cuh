@@ -373,6 +373,20 @@ __device__ __forceinline__ uint32_t segment_of(const uint32_t *seg_off, uint32_t
   return lo;
 }
 
+// The same by a warp (every lane calls it and gets it), 32 probes a step.
+__device__ __forceinline__ uint32_t warp_segment_of(const uint32_t *seg_off, uint32_t S, uint32_t j) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t lo = 0, n = S;  // seg_off[lo] <= j; candidates [lo, lo + n)
+  while (n > 1) {
+    const uint32_t step = (n + 31) / 32, x = lane * step;
+    const bool le = x < n && __ldg(seg_off + lo + x) <= j;
+    const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, le));  // lane 0 always holds
+    lo += k * step;
+    n = n - k * step < step ? n - k * step : step;
+  }
+  return lo;
+}
+
 // Stable rank of digit d among the lanes of a warp, plus the warp's running
 // per-digit count. Peers holding the same digit are found with a
 // shared-memory atomicOr mask (on GB300 about 2.7x the rate of eight

@@ -24,11 +24,15 @@
 namespace gbsa {
 
 constexpr int PACK_BLOCK = 256;
-// Keys of at least this many characters take the sliding fast path (for
-// short keys the per-key loads are already few, and the warp-strided stores
-// of the general path coalesce better: measured 2.89 vs 3.35 ms for 8-char
-// keys at 2^28; 33.9 vs 27.8 ms for 32-char keys at 2^31).
-constexpr uint32_t PACK_SLIDE_MIN = 16;
+// Keys of at least this many characters, in texts long enough for blocks of
+// 4096 keys to fill the GPU, take the sliding fast path; for 8-character keys
+// the per-key loads are few, and the warp-strided stores of the general path
+// coalesce better (2.89 vs 3.35 ms at 2^28). Measured, general against
+// sliding: 12-character keys at 2^20 20.7 / 25.0 us, 2^24 166 / 108 us;
+// 9-character keys at 2^20 23 / 27 us, 2^23 103 / 74 us; 32-character keys at
+// 2^31 33.9 / 27.8 ms.
+constexpr uint32_t PACK_SLIDE_MIN = 9, PACK_SLIDE_ALWAYS = 16;
+constexpr uint32_t PACK_SLIDE_N = 1u << 22;
 
 // Digit histograms of one key (warp-aggregated when a warp shares a digit).
 // With top_only, only the most significant digit's (the others follow from
@@ -52,7 +56,7 @@ __device__ __forceinline__ void pack_hist(uint32_t (*s_hist)[RADIX], const Digit
 // are accumulated here as well, so the sort needs no separate read of the
 // keys.
 //
-// Fast path (keys of PACK_SLIDE_MIN or more characters, the block's keys
+// Fast path (16 keys per thread, the block's keys
 // all in one text's non-tail range, where index j holds position j - t and
 // every key has c0 characters): the text
 // window is staged once in shared memory as dense codes, and each thread
@@ -81,14 +85,17 @@ __global__ void __launch_bounds__(PACK_BLOCK) k_pack(PackArgs a) {
   for (int x = tid; x < MAX_PASSES * RADIX; x += PACK_BLOCK) (&s_hist[0][0])[x] = 0;
   const uint64_t j0 = (uint64_t)blockIdx.x * PACK_SPAN;
   const uint64_t jl = min(j0 + PACK_SPAN, (uint64_t)a.N) - 1;
-  if (tid < 2) s_seg[tid] = a.S > 1 ? segment_of(a.seg_off, a.S, (uint32_t)(tid == 0 ? j0 : jl)) : 0u;
+  if (tid < 64) {  // a warp each
+    const uint32_t s = a.S > 1 ? warp_segment_of(a.seg_off, a.S, (uint32_t)(tid < 32 ? j0 : jl)) : 0u;
+    if (lane == 0) s_seg[tid >> 5] = s;
+  }
   __syncthreads();
   const uint32_t s_lo = s_seg[0], s_hi = s_seg[1];
 
   // Fast-path test (block-uniform).
   bool fast = false;
   uint32_t f_off = 0, f_t = 0;
-  if (s_lo == s_hi && a.c0 >= PACK_SLIDE_MIN && a.c0 <= 64) {
+  if (ITEMS == 16 && s_lo == s_hi && a.c0 <= 64) {
     f_off = __ldg(a.seg_off + s_lo);
     const uint32_t len = __ldg(a.seg_off + s_lo + 1) - f_off;
     f_t = len < a.c0 - 1 ? len : a.c0 - 1;
@@ -261,7 +268,7 @@ cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream) {
     }
     return cudaGetLastError();
   }
-  if (a.c0 >= PACK_SLIDE_MIN) {
+  if (a.c0 >= PACK_SLIDE_ALWAYS || (a.c0 >= PACK_SLIDE_MIN && a.N >= PACK_SLIDE_N)) {
     const uint64_t span = PACK_BLOCK * 16;
     k_pack<16><<<(unsigned)((a.N + span - 1) / span), PACK_BLOCK, 0, stream>>>(a);
   } else {
