@@ -148,7 +148,7 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-KERNEL_SOURCES = {"onesweep": "k_sort.cu", "refine": "k_refine.cu", "rename": "k_rename.cu",
+KERNEL_SOURCES = {"onesweep": "k_sort.cu", "refine": "k_refine.cu", "rename": "k_local.cu",
                   "bucket": "k_bucket.cu",
                   "scatter": "k_refine.cu", "apply": "k_refine.cu", "pack": "k_pack.cu"}
 

@@ -18,7 +18,7 @@
  *  - Pointers are DEVICE pointers unless the parameter says HOST.
  *  - All GPU work is ordered on `stream` (a cudaStream_t; NULL = the legacy
  *    default stream). The call returns after the result is complete on the
- *    device: it synchronises `stream` once per doubling round to read the
+ *    device: it waits for `stream` once or twice per doubling round to read the
  *    number of suffixes still active.
  *  - The caller owns every buffer it passes. The library never frees them
  *    and keeps no pointer to them after returning.
@@ -87,7 +87,7 @@ typedef struct {
   uint32_t paper_names;
   /* Tile shape of the small-group refine of rounds >= 1 (threads per block
    * x items per tile): 0 = automatic, 1 = 128 x 1024, 2 = 256 x 2048,
-   * 3 = 256 x 4096, 4 = 256 x 1024. Groups of up to half a tile are refined
+   * 3 = 256 x 4096, 4 = 256 x 1024. Groups of up to 384, 512, 2048 and 512 items are refined
    * inside one tile; larger ones take the global radix sort. Any other
    * value: SA_ERR_INVALID_ARG. */
   uint32_t refine_shape;
@@ -475,7 +475,9 @@ sa_status sa_bwt(const uint8_t *text, uint64_t n, const uint32_t *sa, uint8_t *b
  * The other direct consumer of SA named as future work (Section 3):
  * lcp_out[0] = 0 and, for j >= 1, lcp_out[j] = the length of the longest
  * common prefix of the suffixes sa[j-1] and sa[j] (Section 2's order).
- * Computed in the permuted form of Kasai et al.'s algorithm (Phi, PLCP).
+ * Neighbours are compared directly where a sample finds their common
+ * prefixes short, else in the permuted form of Kasai et al.'s algorithm (Phi,
+ * PLCP); the choice is made on the device.
  * text      : DEVICE, n bytes, read only.
  * sa        : DEVICE, n uint32, the suffix array of text (sa_build).
  * lcp_out   : DEVICE, n uint32, written.

@@ -8,8 +8,10 @@
 //
 //   k_refine (one tile = whole groups whose starts fall in the tile's
 //   window): load the tile's (g, i') from the active
-//   list, gather the partner names r2 = ISA[i' + h] + 1 (Algorithm 4), sort
-//   by (local group, r2) with a radix sort in shared memory, then rename
+//   list, gather the partner names r2 = ISA[i' + h] + 1 (Algorithm 4), order
+//   by (local group, r2) -- by comparisons inside small groups, around each
+//   larger group's first partner name (refine_pivot), or with a radix sort in
+//   shared memory -- then rename
 //   (CmpName + max PrefixSum inside the tile; NameDiscarding's
 //   r + (subgroup start - group start)), write SA for suffixes that became
 //   unique, compact the survivors into the next active list and queue every
@@ -23,7 +25,7 @@
 //   k_scatter_updates applies the queued updates after every gather of the
 //   round has finished.
 //
-// Groups larger than REFINE_SMALL_MAX take the global path: k_gather_large
+// Groups larger than the tile shape's limit (REFINE_SHAPE) take the global path: k_gather_large
 // builds (large-group ordinal, r2) keys, the one-sweep radix sort orders
 // them and k_rename renames them (after the refine, so its direct ISA
 // writes come after every gather).

@@ -241,7 +241,7 @@ struct CollectArgs {
 cudaError_t launch_need_collect(const CollectArgs &a, int num_sms, cudaStream_t stream);
 
 // ---- rounds >= 1: small-group refine and large-group path (k_refine.cu) --
-// Groups of up to REFINE_SMALL_MAX members are refined inside one tile
+// Groups of up to the shape's `small` members are refined inside one tile
 // (gather, shared-memory sort, rename, compaction); larger ones go through
 // the global radix sort and k_rename.
 // Tile shapes of the refine: threads per block, items one tile can hold, and
