@@ -1408,15 +1408,19 @@ struct Build {
     double best = P + RENAME_COST;
     uint32_t split = 0;
     // Characters by the logarithm of their text's length.
-    double mass[33] = {}, count[33] = {}, log_len[33] = {};
+    uint64_t chars_of[33] = {}, texts_of[33] = {};
     for (uint32_t k = 0; k < S; ++k) {
-      const uint64_t len = off[k + 1] - off[k];
-      if (!len) continue;
-      mass[bits_for(len) - 1] += (double)len / (double)N;
-      count[bits_for(len) - 1] += 1.0;
+      const uint32_t len = off[k + 1] - off[k];
+      const int l = len ? 31 - __builtin_clz(len) : 32;
+      chars_of[l] += len;
+      ++texts_of[l];
     }
-    for (int l = 0; l < 33; ++l)
-      if (count[l] > 0.0) log_len[l] = std::log2(mass[l] * (double)N / count[l]);
+    double mass[33] = {}, log_len[33] = {};
+    for (int l = 0; l < 32; ++l) {
+      if (!texts_of[l]) continue;
+      mass[l] = (double)chars_of[l] / (double)N;
+      log_len[l] = std::log2((double)chars_of[l] / (double)texts_of[l]);
+    }
     for (uint32_t p = 1; p * RADIX_BITS < bits0; ++p) {
       const uint32_t T = p * RADIX_BITS;
       const double chars = T > segbits ? (double)(T - segbits) / b : 0.0;
