@@ -90,3 +90,15 @@ def test_needed_entries(gb, orc, h0, copy):
     sa, _, st, _ = gb.sa_build_ex(torch.from_numpy(t).cuda(), h0_chars=h0)
     assert st["rounds"] > 5
     assert orc.check_sa(t, u32(sa)) == (0, -1)
+
+
+@pytest.mark.parametrize("count,size", [(3, 3000), (4, 90001), (20, 200003)])
+def test_batch_of_unlike_texts(gb, orc, count, size):
+    """Texts of four letters beside texts of many: more top digits are sorted
+    than the counts of the whole batch ask for."""
+    import torch
+    texts = [gen.text("zipf" if k % 2 else "dna", 40 + k, size - 7 * k) for k in range(count)]
+    off = np.concatenate([[0], np.cumsum([x.size for x in texts])]).astype(np.uint64)
+    got = u32(gb.sa_build_batched(torch.from_numpy(np.concatenate(texts)).cuda(), off))
+    for k, x in enumerate(texts):
+        assert np.array_equal(got[int(off[k]):int(off[k + 1])], orc.pd_sa(x)[0]), k
