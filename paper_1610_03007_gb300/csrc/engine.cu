@@ -1817,7 +1817,9 @@ struct Build {
       if (s != SA_OK) return s;
       bytes += 8ull * N;
     }
-    if (prof) {
+    // The SA is complete with the last round's readback; the ISA, and the
+    // trace of a text resolved in round 0, are written after it.
+    if (prof || isa_out || want_trace) {
       CK(cudaStreamSynchronize(st));
       s = flush(0, 0);
       if (s != SA_OK) return s;
@@ -2018,6 +2020,7 @@ sa_status build_single(const uint8_t *text, uint64_t n, uint32_t *sa_out, uint32
   if (n == 1) {
     if (cudaMemsetAsync(sa_out, 0, 4, st) != cudaSuccess) return SA_ERR_CUDA;
     if (isa_out && cudaMemsetAsync(isa_out, 0, 4, st) != cudaSuccess) return SA_ERR_CUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return SA_ERR_CUDA;
     if (stats) stats->rounds = 1;
     return SA_OK;
   }
