@@ -245,10 +245,25 @@ def _torch():
     return torch
 
 
-def _stream(stream) -> int:
+def _torch_stream(stream):
+    """`stream` (anything with a cuda_stream handle) as a torch stream; None
+    for torch's current one."""
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is None or isinstance(stream, torch.cuda.Stream):
+        return stream
+    return torch.cuda.ExternalStream(stream.cuda_stream)
+
+
+def _stream(stream) -> int:
+    """Handle of the stream a call runs on. One that is not torch's current
+    stream waits for it: buffers were allocated, filled or made contiguous
+    there."""
+    cur = _torch().cuda.current_stream()
+    if stream is None:
+        return cur.cuda_stream
+    if stream.cuda_stream != cur.cuda_stream:
+        _torch_stream(stream).wait_stream(cur)
+    return stream.cuda_stream
 
 
 def _check(status: int, where: str):
@@ -456,7 +471,8 @@ def sa_bwt(text, sa, stream=None):
     prim = torch.zeros(1, dtype=torch.int64, device=t.device)
     _check(lib.sa_bwt(t.data_ptr() if n else None, n, sa.data_ptr() if n else None,
                       bwt.data_ptr(), prim.data_ptr(), _stream(stream)), "sa_bwt")
-    return bwt, int(prim.item())
+    with torch.cuda.stream(_torch_stream(stream)):  # the read follows the kernel that writes it
+        return bwt, int(prim.item())
 
 
 def sa_build_dc3(text, trace=False, stream=None):
@@ -533,6 +549,9 @@ def sa_lcp(text, sa, workspace=None, stream=None):
     _check(lib.sa_lcp(t.data_ptr() if n else None, n, sa.data_ptr() if n else None,
                       lcp.data_ptr() if n else None, ws_ptr, ws_bytes, _stream(stream)),
            "sa_lcp")
+    if stream is not None and n:  # the call does not wait: keep its buffers from other uses
+        for x in (t, sa, workspace, lcp):
+            x.record_stream(_torch_stream(stream))
     return lcp
 
 
