@@ -88,7 +88,8 @@ typedef struct {
   /* Tile shape of the small-group refine of rounds >= 1 (threads per block
    * x items per tile): 0 = automatic, 1 = 128 x 1024, 2 = 256 x 2048,
    * 3 = 256 x 4096, 4 = 256 x 1024. Groups of up to 384, 512, 2048 and 512 items are refined
-   * inside one tile; larger ones take the global radix sort. Any other
+   * inside one tile (512 and 1024 in the first two shapes where many suffixes
+   * are in groups between); larger ones take the global radix sort. Any other
    * value: SA_ERR_INVALID_ARG. */
   uint32_t refine_shape;
   /* Keys per thread of the one-sweep radix pass (tile = 256 x this):

@@ -7,7 +7,8 @@ Four knobs of a build are picked by measurement rather than fixed:
   barriers, smaller ones fit more blocks per SM.
 - ``refine_shape`` -- threads x items of the small-group refine (128 x 1024,
   256 x 2048, 256 x 4096, 256 x 1024). It also sets the segment threshold:
-  groups of up to half a tile are refined inside one block, larger ones take
+  groups of up to 384, 512, 2048 and 512 items (half a tile where many suffixes
+  are in groups between) are refined inside one block, larger ones take
   the global radix sort.
 - ``h0_chars`` -- characters per initial key (0: as many as fit in 64
   bits). Fewer characters mean fewer key bits, so fewer radix passes in

@@ -37,7 +37,7 @@ struct RoundCounts {
   uint32_t m_s, g_s;        // survivors / groups written by the refine
   uint32_t m_l, g_l;        // survivors / groups written by the rename
   uint32_t upd;             // deferred ISA updates queued by the refine
-  uint32_t pad;
+  uint32_t mid;             // classify: items of large groups that a refine tile could hold
   unsigned long long large; // classify: (large groups << 32) | large items
 };
 

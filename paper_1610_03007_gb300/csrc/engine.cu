@@ -370,7 +370,7 @@ struct PrefixModel {
 
 struct HostCtrl {
   uint32_t error, err_where, passes, pass_mask;
-  uint32_t m_s, g_s, m_l, g_l, upd, pad;
+  uint32_t m_s, g_s, m_l, g_l, upd, mid;
   unsigned long long large;
   uint32_t zero[4];
   uint32_t m_next() const { return m_s + m_l; }
@@ -418,7 +418,7 @@ struct Build {
   uint64_t bytes = 0;
   uint32_t launches = 0;
   uint32_t naming = NAMES_RETAIN;
-  uint32_t shape = 0, nominal = 512;  // refine tile shape and window
+  uint32_t shape = 0, nominal = 512, small = 512;  // refine tile shape, window, largest group
   uint32_t sort_items = SORT_ITEMS_DEFAULT;  // keys per thread of the radix pass
   uint32_t bucket_min = BUCKET_MIN;  // pending ISA writes that are bucketed first
   uint32_t mult = 2;  // a: names ranked per round (2: doubling, 4: quadrupling)
@@ -728,7 +728,8 @@ struct Build {
     ca.lold = lold;
     ca.tfirst = tfirst;
     ca.nominal = nominal;
-    ca.small = REFINE_SHAPE[shape].small;
+    ca.small = small;
+    ca.cap = REFINE_SHAPE[shape].cap;
     ca.max_groups = L.max_groups;
     ca.max_tiles = L.max_tiles;
     ca.ctrl = ctrl;
@@ -959,6 +960,7 @@ struct Build {
     rf.tfirst = tfirst;
     rf.m = m1;
     rf.shape = shape;
+    rf.small = small;
     rf.tiles = (m1 + nominal - 1) / nominal;
     rf.W = W;
     rf.mult = 2;
@@ -1045,7 +1047,8 @@ struct Build {
     ca.lold = lold;
     ca.tfirst = tfirst;
     ca.nominal = nominal;
-    ca.small = REFINE_SHAPE[shape].small;
+    ca.small = small;
+    ca.cap = REFINE_SHAPE[shape].cap;
     ca.max_groups = L.max_groups;
     ca.max_tiles = L.max_tiles;
     ca.ctrl = ctrl;
@@ -1191,6 +1194,27 @@ struct Build {
   bool position_order_wanted(uint32_t m) const {
     if (opt.group_order) return opt.group_order == 1;
     return N >= (1ull << 24) && m >= N / 16;
+  }
+
+  // Half a tile as the refine's window and largest group, for the rest of
+  // the build, where many of the suffixes active after round 0 are in groups
+  // that are above the shape's own limit but fit a tile (REFINE_HALF_SHARE):
+  // they are refined in tiles then, at once or after they have split once.
+  // With again, the list is classified again and hc.large re-read.
+  sa_status refine_limits(int cur, HostCtrl &hc, bool again) {
+    const uint32_t half = REFINE_SHAPE[shape].cap / 2;
+    if (hc.mid <= hc.m_next() / REFINE_HALF_SHARE || small == half) return SA_OK;
+    small = nominal = half;
+    if (!again) return SA_OK;
+    CK(cudaMemsetAsync(&ctrl->rc.large, 0, sizeof(ctrl->rc.large), st));
+    sa_status s = classify(cur, hc.g_next(), 0);
+    if (s != SA_OK) return s;
+    HostCtrl h2{};
+    s = read_ctrl(h2);
+    if (s != SA_OK) return s;
+    hc.large = h2.large;
+    bytes += 8ull * hc.g_next();
+    return flush(0, 0);
   }
 
   // The groups of the active list `cur` (hc: its counts) copied to the
@@ -1541,7 +1565,8 @@ struct Build {
                       items_ok(opt.sort_items), items_ok(tuned.sort_items));
     shape = pick(opt.refine_shape, tuned.refine_shape, 1, shape_ok(opt.refine_shape),
                  shape_ok(tuned.refine_shape)) - 1;
-    nominal = REFINE_SHAPE[shape].window();
+    small = REFINE_SHAPE[shape].small;
+    nominal = REFINE_SHAPE[shape].cap - small;
     bucket_min = pick(opt.bucket_min, tuned.bucket_min, BUCKET_MIN, true, true);
     const uint32_t h0 = pick(opt.h0_chars, tuned.h0_chars, 0, true, true);
     uint32_t c0 = (64 - segbits) / b;
@@ -1658,7 +1683,10 @@ struct Build {
       settle(hc);
     }
     if (want_trace) CK(cudaMemcpyAsync(opt.trace_isa, isa, N * 4, cudaMemcpyDeviceToDevice, st));
-    if (hc.m_next() > 0 && position_order_wanted(hc.m_next())) {
+    const bool reorder = hc.m_next() > 0 && position_order_wanted(hc.m_next());
+    s = refine_limits(cur, hc, !reorder);
+    if (s != SA_OK) return s;
+    if (reorder) {
       // The later rounds read partner names through the ISA: groups in
       // position order make those reads of neighbouring groups neighbours.
       s = reorder_groups(cur, hc);
@@ -1761,6 +1789,7 @@ struct Build {
       rf.m = m;
       rf.G = G;
       rf.shape = shape;
+      rf.small = small;
       rf.tiles = (m + nominal - 1) / nominal;
       rf.h = (uint32_t)h;
       rf.W = W;

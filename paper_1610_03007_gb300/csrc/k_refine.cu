@@ -25,7 +25,7 @@
 //   k_scatter_updates applies the queued updates after every gather of the
 //   round has finished.
 //
-// Groups larger than the tile shape's limit (REFINE_SHAPE) take the global path: k_gather_large
+// Groups larger than the limit of the build's tiles (REFINE_SHAPE) take the global path: k_gather_large
 // builds (large-group ordinal, r2) keys, the one-sweep radix sort orders
 // them and k_rename renames them (after the refine, so its direct ISA
 // writes come after every gather).
@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(256) k_classify(ClassifyArgs a) {
           a.loff[k] = off;
           a.lbase[k] = a.ghead[x] - off;
           a.lold[k] = name;
+          if (size <= a.cap) atomicAdd(&a.ctrl->rc.mid, size);
         }
       }
       if (x <= tiles) a.tfirst[x] = lower_bound_u32(a.gstart, G, (uint32_t)x * a.nominal);
@@ -262,8 +263,8 @@ template <int BLOCK, int CAP>
 struct RfCfg {
   static constexpr int WARPS = BLOCK / 32;
   static constexpr int ITEMS = CAP / BLOCK;       // slots per thread
-  static constexpr int SMALL = rf_small(BLOCK, CAP);   // largest small group
-  static constexpr int MAXG = (CAP - SMALL) / 2 + 1;   // starts in a window: groups have >= 2 members
+  // Starts in the widest window: groups have >= 2 members.
+  static constexpr int MAXG = (CAP - rf_small(BLOCK, CAP)) / 2 + 1;
   static constexpr int GPT = (MAXG + BLOCK - 1) / BLOCK;  // groups per thread
   static constexpr int DPT = RADIX / BLOCK;       // digits per thread in the digit scan
   static constexpr int SEGS = CAP / 32;           // rows of 32 items
@@ -910,9 +911,10 @@ __device__ __forceinline__ bool refine_pivot(RfSmem<BLOCK, CAP, false> &S, const
   return true;
 }
 
-// One refine tile (whole groups whose starts fall in the tile's window).
+// One refine tile (whole groups whose starts fall in the tile's window, of up
+// to SMALL members: as an argument of the launch it cost pairs 2.5 %).
 // Every thread of the block calls it; all returns are block-uniform.
-template <int BLOCK, int CAP, bool WIDE>
+template <int BLOCK, int CAP, bool WIDE, int SMALL>
 __device__ __forceinline__ void refine_tile(RfSmem<BLOCK, CAP, WIDE> &S, const RefineArgs &a,
                                             const uint32_t tile, const uint32_t h) {
   using C = RfCfg<BLOCK, CAP>;
@@ -951,7 +953,7 @@ __device__ __forceinline__ void refine_tile(RfSmem<BLOCK, CAP, WIDE> &S, const R
       S.gname[lg] = __ldg(a.gname + g);
       S.ghead[lg] = __ldg(a.ghead + g);
       const uint32_t size = e - s;
-      if (size <= (uint32_t)C::SMALL)
+      if (size <= (uint32_t)SMALL)
         sz[r] = size;
       else
         mybig = 1;
@@ -1308,14 +1310,14 @@ renamed_order:
 // Blocks take tiles blockIdx.x, + gridDim.x, ... (tiles share nothing, so
 // any grid works); in device-driven rounds the tile count and h come from
 // the round state.
-template <int BLOCK, int CAP, bool WIDE, bool PERSIST>
+template <int BLOCK, int CAP, bool WIDE, bool PERSIST, int SMALL>
 __global__ void __launch_bounds__(BLOCK, (CAP / BLOCK > 8 ? 512 : 1024) / BLOCK)
     k_refine(RefineArgs a) {
   using Sm = RfSmem<BLOCK, CAP, WIDE>;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   Sm &S = *reinterpret_cast<Sm *>(smem_raw);
   if constexpr (!PERSIST) {  // one tile per block (host-driven rounds)
-    refine_tile<BLOCK, CAP, WIDE>(S, a, blockIdx.x, a.h);
+    refine_tile<BLOCK, CAP, WIDE, SMALL>(S, a, blockIdx.x, a.h);
   } else {
     uint32_t tiles = a.tiles, h = a.h;
     if (a.rs) {
@@ -1324,29 +1326,38 @@ __global__ void __launch_bounds__(BLOCK, (CAP / BLOCK > 8 ? 512 : 1024) / BLOCK)
       h = a.rs->h;
     }
     for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-      refine_tile<BLOCK, CAP, WIDE>(S, a, tile, h);
+      refine_tile<BLOCK, CAP, WIDE, SMALL>(S, a, tile, h);
       __syncthreads();  // the next tile reuses the shared buffers
     }
   }
 }
 
-template <int BLOCK, int CAP, bool WIDE, bool PERSIST>
+template <int BLOCK, int CAP, bool WIDE, bool PERSIST, int SMALL>
 cudaError_t launch_refine_p(const RefineArgs &a, uint32_t grid, cudaStream_t stream) {
   const int smem = (int)sizeof(RfSmem<BLOCK, CAP, WIDE>);
   cudaError_t e = ensure_smem_attributes(
-      reinterpret_cast<const void *>(&k_refine<BLOCK, CAP, WIDE, PERSIST>), smem, true);
+      reinterpret_cast<const void *>(&k_refine<BLOCK, CAP, WIDE, PERSIST, SMALL>), smem, true);
   if (e != cudaSuccess) return e;
-  k_refine<BLOCK, CAP, WIDE, PERSIST><<<grid, BLOCK, smem, stream>>>(a);
+  k_refine<BLOCK, CAP, WIDE, PERSIST, SMALL><<<grid, BLOCK, smem, stream>>>(a);
   return cudaGetLastError();
 }
 
 // The one-tile-per-block instance unless the round state or a grid cap
 // asks for the looping one (its loop costs the single-tile form registers).
+template <int BLOCK, int CAP, bool WIDE, int SMALL>
+cudaError_t launch_refine_s(const RefineArgs &a, cudaStream_t stream) {
+  if (!a.rs && !a.grid_cap)
+    return launch_refine_p<BLOCK, CAP, WIDE, false, SMALL>(a, a.tiles, stream);
+  const uint32_t grid = a.grid_cap && a.tiles > a.grid_cap ? a.grid_cap : a.tiles;
+  return launch_refine_p<BLOCK, CAP, WIDE, true, SMALL>(a, grid, stream);
+}
+
 template <int BLOCK, int CAP, bool WIDE>
 cudaError_t launch_refine_t(const RefineArgs &a, cudaStream_t stream) {
-  if (!a.rs && !a.grid_cap) return launch_refine_p<BLOCK, CAP, WIDE, false>(a, a.tiles, stream);
-  const uint32_t grid = a.grid_cap && a.tiles > a.grid_cap ? a.grid_cap : a.tiles;
-  return launch_refine_p<BLOCK, CAP, WIDE, true>(a, grid, stream);
+  constexpr int OWN = rf_small(BLOCK, CAP);
+  if (a.small == (uint32_t)OWN) return launch_refine_s<BLOCK, CAP, WIDE, OWN>(a, stream);
+  if (a.small == CAP / 2) return launch_refine_s<BLOCK, CAP, WIDE, CAP / 2>(a, stream);
+  return cudaErrorInvalidValue;
 }
 
 template <bool WIDE>

@@ -241,26 +241,33 @@ struct CollectArgs {
 cudaError_t launch_need_collect(const CollectArgs &a, int num_sms, cudaStream_t stream);
 
 // ---- rounds >= 1: small-group refine and large-group path (k_refine.cu) --
-// Groups of up to the shape's `small` members are refined inside one tile
+// Groups of up to `small` members are refined inside one tile
 // (gather, shared-memory sort, rename, compaction); larger ones go through
 // the global radix sort and k_rename.
 // Tile shapes of the refine: threads per block, items one tile can hold, and
 // the largest small group. Tile t owns the groups whose starts fall in
 // [t, t+1) * (cap - small) of the active list, so a tile's groups always fit.
 // The first two shapes' wider windows spread a tile's fixed work over more
-// items; groups above the limit cost more in the global sort. Refine of the
-// 2^28 repeated Zipf text (groups of about 250) with 256 x 2048 tiles and
-// groups of up to 1024, 768, 640, 512: 51.3, 46.4, 44.8, 43.6 ms; of 2^28
-// Markov DNA (pairs) with 128 x 1024 and up to 512, 384, 256: 3.78, 3.39,
-// 4.00 ms.
+// items where few groups are above `small`, which cost more in the global
+// sort. Refine of the 2^28 repeated Zipf text (groups of about 250) with 256 x
+// 2048 tiles and groups of up to 1024, 768, 640, 512: 51.3, 46.4, 44.8, 43.6
+// ms; of 2^28 Markov DNA (pairs) with 128 x 1024 and up to 512, 384, 256:
+// 3.78, 3.39, 4.00 ms. Where more than one active suffix in REFINE_HALF_SHARE
+// is in a group above `small` that a tile can hold, the build takes half a tile
+// as window and limit (Build::refine_limits). Builds of 2^27 characters,
+// copies of a Zipf block 600, 800, 1000, 1500 times: 87.7, 93.1, 97.4, 101.0 ms
+// with groups of up to 512, 40.8, 42.0, 42.8, 96.1 with 1024; of a DNA block
+// 400, 500, 600 times 49.8, 72.2, 76.8 with 384, 39.5, 39.3, 69.0 with 512. The
+// share at which both take the same time: Zipf 800 copies beside 250 0.08,
+// DNA 450 beside 100 0.075. Groups above the tile gain nothing (5000 copies).
 struct RefineShape {
   uint32_t block, cap, small;
-  constexpr uint32_t window() const { return cap - small; }
 };
 constexpr int REFINE_SHAPES = 4;
 constexpr RefineShape REFINE_SHAPE[REFINE_SHAPES] = {
     {128, 1024, 384}, {256, 2048, 512}, {256, 4096, 2048}, {256, 1024, 512}};
 constexpr uint32_t REFINE_MIN_NOMINAL = 256;  // least window and least small (buffer sizing)
+constexpr uint32_t REFINE_HALF_SHARE = 12;
 
 // Names of groups. A name may be any rank inside the group's SA interval:
 // intervals are disjoint and ordered, so such names respect the order of
@@ -283,6 +290,7 @@ struct ClassifyArgs {
                                        // list, head - start, name
   uint32_t *tfirst;         // first group of each refine tile (tiles + 1 entries)
   uint32_t nominal, small;  // refine tile window; the largest small group
+  uint32_t cap;             // items one tile can hold: rc.mid counts those of groups in (small, cap]
   uint32_t max_groups;      // upper bound of G (buffer capacity)
   uint32_t max_tiles;       // upper bound of tiles (buffer capacity - 1)
   Ctrl *ctrl;               // reads rc.m_s + rc.m_l, rc.g_s + rc.g_l; adds to rc.large
@@ -343,6 +351,7 @@ struct RefineArgs {
   uint32_t naming;          // NamingRule
   const uint32_t *tfirst;   // tiles + 1 entries
   uint32_t shape;           // index into REFINE_SHAPE
+  uint32_t small;           // largest small group (as classified)
   uint32_t m, G, tiles;
   uint32_t h, W;
   uint32_t mult;            // a: names of i' + h .. i' + (a-1)h are ranked (2, 3, 4)
