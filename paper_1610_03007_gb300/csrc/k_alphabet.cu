@@ -9,8 +9,18 @@
 // an upload of the codes nor a copy kernel of its own stands on a small
 // text's critical path.
 //
+// The counts say nothing of repeats (copies of a block, words), which make
+// buckets of equal key bits large however many digits are sorted. So one more
+// block draws `samples` positions, sorts the prefixes there and counts, for 1 to
+// SAMPLE_CHARS characters, the pairs and triples that agree in them: the mean
+// bucket size and its spread, as they are. It works beside the counting
+// blocks, on bytes, which need no codes. (1024 positions as a step of the last
+// block, on codes, took 18 us.)
+//
 // Bound: HBM read of n bytes; 16-byte vector loads, per-warp privatised
 // shared-memory counters, one global atomic per bin and block.
+#include <algorithm>
+
 #include "launch.h"
 
 namespace gbsa {
@@ -18,12 +28,118 @@ namespace gbsa {
 constexpr int HIST_BLOCK = 512;
 constexpr int HIST_COPIES = HIST_BLOCK / 32;  // one private histogram per warp
 
-__global__ void __launch_bounds__(HIST_BLOCK)
-k_byte_histogram(AlphabetArgs a) {
+// The 8 characters at pos, first character on top, zeros from `end` on.
+__device__ __forceinline__ uint64_t prefix_at(const uint8_t *text, uint64_t n, uint64_t pos,
+                                              uint64_t end) {
+  const uintptr_t at = (uintptr_t)(text + pos), a0 = at & ~(uintptr_t)7;
+  const uint32_t skip = (uint32_t)(at - a0) * 8u;
+  uint64_t key = 0;
+  if (a0 >= (uintptr_t)text && a0 + 16 <= (uintptr_t)(text + n)) {
+    const unsigned long long *w = reinterpret_cast<const unsigned long long *>(a0);
+    const uint64_t w0 = __ldg(w), w1 = __ldg(w + 1);
+    const uint64_t v = skip ? (w0 >> skip) | (w1 << (64 - skip)) : w0;
+    key = ((uint64_t)__byte_perm((uint32_t)v, 0u, 0x0123) << 32) |
+          __byte_perm((uint32_t)(v >> 32), 0u, 0x0123);
+  } else {  // the text's first and last bytes
+    for (uint32_t i = 0; i < 8; ++i) key = (key << 8) | (pos + i < n ? text[pos + i] : 0u);
+  }
+  return end - pos < 8 ? key & (~0ull << (8 * (8 - (end - pos)))) : key;
+}
+
+// One block: `samples` prefixes (a power of two, at least HIST_BLOCK) below
+// their text's number (textbits), sorted in `keys`.
+__device__ __forceinline__ void sample_prefixes(const AlphabetArgs &a, uint64_t *keys,
+                                                uint32_t textbits) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, s = a.samples;
+  const uint32_t *offsets = a.offsets;
+  if (a.S > 1 && a.S + 1 + 2 * s <= HIST_COPIES * RADIX) {  // searched in shared memory
+    uint32_t *copy = reinterpret_cast<uint32_t *>(keys + s);
+    for (uint32_t i = tid; i <= a.S; i += HIST_BLOCK) copy[i] = a.offsets[i];
+    offsets = copy;
+    __syncthreads();
+  }
+  for (uint32_t i = tid; i < s; i += HIST_BLOCK) {
+    // Evenly spread, shifted at random: a period of the text must not show.
+    uint32_t r = i * 0x9E3779B9u;
+    r = (r ^ (r >> 16)) * 0x85EBCA6Bu;
+    r ^= r >> 13;
+    const uint64_t x = ((uint64_t)i * a.n + (((uint64_t)r * a.n) >> 32)) / s;
+    uint64_t end = a.n, text = 0;
+    if (a.S > 1) {
+      uint32_t lo = 0, hi = a.S - 1;  // the last text with an offset <= x
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (offsets[mid] <= x)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+      end = offsets[lo + 1];
+      text = (uint64_t)lo << (64 - textbits);
+    }
+    keys[i] = text | (prefix_at(a.text, a.n, x, end) >> textbits);
+  }
+  __syncthreads();
+  // Bitonic; the steps inside rows of 32 by shuffles.
+  for (uint32_t k0 = 32; k0 <= s; k0 <<= 1) {
+    for (uint32_t j = k0 >> 1; j >= 32; j >>= 1) {
+      for (uint32_t i = tid; i < s / 2; i += HIST_BLOCK) {
+        const uint32_t lo = 2 * i - (i & (j - 1)), hi = lo + j;
+        const uint64_t p = keys[lo], q = keys[hi];
+        if ((p > q) == ((lo & k0) == 0)) {
+          keys[lo] = q;
+          keys[hi] = p;
+        }
+      }
+      __syncthreads();
+    }
+    for (uint32_t i = tid; i < s; i += HIST_BLOCK) {
+      uint64_t p = keys[i];
+      for (uint32_t k = k0 == 32 ? 2 : k0; k <= k0; k <<= 1) {
+        for (uint32_t j = min(k >> 1, 16u); j > 0; j >>= 1) {
+          const uint64_t q = __shfl_xor_sync(0xffffffffu, p, j);
+          const bool least = ((lane & j) == 0) == ((i & k) == 0);
+          p = (q < p) == least ? q : p;
+        }
+      }
+      keys[i] = p;
+    }
+    __syncthreads();
+  }
+}
+
+// One warp: the pairs and triples of the sorted keys that agree in their top
+// `bits`. A key agrees with every one from its group's head on.
+__device__ __forceinline__ void count_agreeing(const uint64_t *keys, uint32_t s, uint32_t bits,
+                                               uint32_t *pairs_out, unsigned long long *triples_out) {
+  const uint32_t lane = threadIdx.x & 31, R = 64 - bits;
+  uint32_t first = 0;  // the last head so far
+  unsigned long long pairs = 0, triples = 0;
+  for (uint32_t i0 = 0; i0 < s; i0 += 32) {
+    const uint32_t i = i0 + lane;
+    const bool head = i == 0 || ((keys[i] ^ keys[i - 1]) >> R) != 0;
+    const uint32_t H = __ballot_sync(0xffffffffu, head), m = H & (lanemask_lt() | (1u << lane));
+    const unsigned long long before = i - (m ? i0 + 31 - __clz(m) : first);
+    pairs += before;
+    triples += before * (before - 1) / 2;
+    if (H) first = i0 + 31 - __clz(H);
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    pairs += __shfl_xor_sync(0xffffffffu, pairs, d);
+    triples += __shfl_xor_sync(0xffffffffu, triples, d);
+  }
+  if (lane == 0) {
+    *pairs_out = (uint32_t)pairs;
+    *triples_out = triples;
+  }
+}
+
+// Block `block` of `blocks` adds its share of the text to the counts.
+__device__ __forceinline__ void count_bytes(const AlphabetArgs &a, uint32_t (*s_hist)[RADIX],
+                                            uint32_t block, uint32_t blocks) {
   const uint8_t *__restrict__ text = a.text;
   const uint64_t n = a.n;
-  uint32_t *hist = a.hist;
-  __shared__ uint32_t s_hist[HIST_COPIES][RADIX];
   for (int x = threadIdx.x; x < HIST_COPIES * RADIX; x += HIST_BLOCK) (&s_hist[0][0])[x] = 0;
   __syncthreads();
   uint32_t *mine = s_hist[threadIdx.x >> 5];
@@ -33,8 +149,8 @@ k_byte_histogram(AlphabetArgs a) {
   if (head > n) head = n;
   const uint64_t body = (n - head) / 16;
   const uint4 *vec = (const uint4 *)(text + head);
-  const uint64_t stride = (uint64_t)gridDim.x * HIST_BLOCK;
-  for (uint64_t v = (uint64_t)blockIdx.x * HIST_BLOCK + threadIdx.x; v < body; v += stride) {
+  const uint64_t stride = (uint64_t)blocks * HIST_BLOCK;
+  for (uint64_t v = (uint64_t)block * HIST_BLOCK + threadIdx.x; v < body; v += stride) {
     uint4 q = __ldg(vec + v);
     uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
@@ -44,7 +160,7 @@ k_byte_histogram(AlphabetArgs a) {
     }
   }
   const uint64_t tail0 = head + body * 16;
-  const uint64_t gtid = (uint64_t)blockIdx.x * HIST_BLOCK + threadIdx.x;
+  const uint64_t gtid = (uint64_t)block * HIST_BLOCK + threadIdx.x;
   if (gtid < head) atomicAdd(&mine[text[gtid]], 1u);
   if (gtid < n - tail0) atomicAdd(&mine[text[tail0 + gtid]], 1u);
   __syncthreads();
@@ -52,7 +168,26 @@ k_byte_histogram(AlphabetArgs a) {
     uint32_t s = 0;
 #pragma unroll
     for (int c = 0; c < HIST_COPIES; ++c) s += s_hist[c][d];
-    if (s) atomicAdd(&hist[d], s);
+    if (s) atomicAdd(&a.hist[d], s);
+  }
+}
+
+__global__ void __launch_bounds__(HIST_BLOCK, 4) k_byte_histogram(AlphabetArgs a) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  uint32_t *hist = a.hist;
+  const uint64_t n = a.n;
+  const uint32_t sampling = a.samples ? 1u : 0u;
+  if (blockIdx.x < sampling) {
+    uint64_t *keys = reinterpret_cast<uint64_t *>(smem_raw);
+    const uint32_t textbits = a.S > 1 ? 32 - __clz(a.S - 1) : 0;
+    sample_prefixes(a, keys, textbits);
+    KeySample *out = reinterpret_cast<KeySample *>(hist + RADIX);
+    const uint32_t w = threadIdx.x >> 5, bits = textbits + 8 * (w + 1);
+    if (w < SAMPLE_CHARS && bits <= 64)
+      count_agreeing(keys, a.samples, bits, &out->pairs[w], &out->triples[w]);
+  } else {
+    count_bytes(a, reinterpret_cast<uint32_t (*)[RADIX]>(smem_raw), blockIdx.x - sampling,
+                gridDim.x - sampling);
   }
   __shared__ uint32_t s_last, s_tmp[HIST_COPIES + 1];
   __syncthreads();
@@ -71,6 +206,7 @@ k_byte_histogram(AlphabetArgs a) {
     a.code[d] = (uint8_t)code;
     if (a.host) a.host[d] = c;
   }
+  if (a.host && d < sizeof(KeySample) / 4) a.host[RADIX + d] = load_volatile_u32(hist + RADIX + d);
   if (d < 2 && a.seg_off) a.seg_off[d] = d ? (uint32_t)n : 0u;
   if (a.host) report_to_host(a.host_flag);
 }
@@ -78,9 +214,10 @@ k_byte_histogram(AlphabetArgs a) {
 cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream) {
   if (a.n == 0) return cudaSuccess;
   uint64_t want = (a.n / 16 + HIST_BLOCK - 1) / HIST_BLOCK;
-  uint64_t cap = (uint64_t)num_sms * 4;
+  uint64_t cap = (uint64_t)num_sms * 4 - (a.samples ? 1 : 0);  // resident at once
   unsigned grid = (unsigned)(want < 1 ? 1 : (want > cap ? cap : want));
-  k_byte_histogram<<<grid, HIST_BLOCK, 0, stream>>>(a);
+  const size_t smem = std::max<size_t>(HIST_COPIES * RADIX * 4, (size_t)a.samples * 8);
+  k_byte_histogram<<<grid + (a.samples ? 1 : 0), HIST_BLOCK, smem, stream>>>(a);
   return cudaGetLastError();
 }
 

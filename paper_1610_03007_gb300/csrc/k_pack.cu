@@ -36,7 +36,7 @@ constexpr uint32_t PACK_SLIDE_N = 1u << 22;
 
 // Digit histograms of one key (warp-aggregated when a warp shares a digit).
 // With top_only, only the most significant digit's (the others follow from
-// it, k_pack_hist_fixup).
+// it, k_sort_plan).
 __device__ __forceinline__ void pack_hist(uint32_t (*s_hist)[RADIX], const DigitSpec &spec,
                                           uint64_t key, bool valid, int lane, bool top_only) {
   const uint32_t nvalid = __popc(__ballot_sync(0xffffffffu, valid));

@@ -36,14 +36,24 @@ cudaError_t launch_copy_words(uint32_t *dst, const uint32_t *src, uint64_t words
 cudaError_t launch_copy_bytes(uint8_t *dst, const uint8_t *src, uint64_t n, cudaStream_t stream);
 
 // ---- step A0: alphabet (k_alphabet.cu) ----------------------------------
+// Of `samples` prefixes: pairs and triples of one text that agree in 1, 2, ..
+// characters (0 beyond what 64 bits hold beside the text's number).
+constexpr uint32_t SAMPLE_MAX = 4096, SAMPLE_CHARS = 8;
+struct KeySample {
+  unsigned long long triples[SAMPLE_CHARS];
+  uint32_t pairs[SAMPLE_CHARS];
+};
 struct AlphabetArgs {
   const uint8_t *text;
   uint64_t n;
-  uint32_t *hist;     // 256 counts (zeroed by the caller), += the text's
+  uint32_t *hist;     // 256 counts (zeroed by the caller), += the text's; then a KeySample
   uint32_t *done;     // blocks finished (zeroed by the caller)
   uint8_t *code;      // out: dense order-preserving code of each byte value
   uint32_t *seg_off;  // out, for one text: {0, n} (NULL otherwise)
-  uint32_t *host;     // out: the counts in pinned host memory, or NULL
+  uint32_t *host;     // out: the counts and the sample in pinned host memory, or NULL
+  uint32_t samples;   // prefixes to draw: 0 or a power of two in [512, SAMPLE_MAX]
+  const uint32_t *offsets;  // S + 1 offsets of a batch (S > 1)
+  uint32_t S;
   uint32_t *host_flag;  // set to 1 after them
 };
 cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream);
@@ -70,7 +80,7 @@ struct PackArgs {
 // keys == NULL (top_only only): only the top digit's histogram (the first
 // radix pass then builds the keys from the text, PassArgs.text). With
 // top_only the counts go to the last of the MAX_PASSES rows, from which
-// launch_pack_fixup derives the rows of the digits in spec.
+// launch_sort_plan derives the rows of the digits in spec.
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t stream);
 
 // ---- step A2: radix sort (k_sort.cu) ------------------------------------
