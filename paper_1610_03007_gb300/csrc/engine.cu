@@ -260,61 +260,57 @@ constexpr double LOCAL_LARGE_LOG2 = 10.3;
 // (k_isa.cu), and from the second on they go through a list that can be
 // bucketed by position (an ISA that the L2 holds is written directly).
 constexpr uint64_t NEED_MIN_N = 1ull << 22, COLLECT_MIN_N = 1ull << 25;
-// The share of a batch's characters that the choice takes to be texts of FEW_BITS
-// per character, where its alphabet is larger: the counts are over the whole
-// batch and hide such texts, whose buckets after too few digits are large.
-// In them only whole characters divide (a few letters have close codes).
-// Measured (builds in ms; chosen by the counts alone, with this, unsplit):
-// half DNA, half Zipf bytes, 4, 8, 14, 48 texts of 10-256 KB 0.38, 0.43, 0.49,
-// 0.79; 0.33, 0.35, 0.42, 0.74; 0.33, 0.36, 0.41, 0.73. What it costs where
-// the texts are alike: Zipf bytes 64 and 256 texts 0.48, 3.11; 0.53, 3.28;
-// 0.59, 3.93, protein 64 and 256 texts 0.27, 2.26; 0.30, 2.60; 0.47, 3.57.
-constexpr double FEW_SHARE = 0.5, FEW_BITS = 2.0;
 // Texts at least this long wait for the gram histogram to model their
 // prefixes by its statistics; shorter ones take the character counts.
 constexpr uint64_t GRAM_MODEL_MIN = 1ull << 22;
 
-// Texts at least this long are sampled (KeySample), with as many positions as
-// the counting blocks take time for: 512, 1024, 2048 positions beside 2^22
-// characters +2.0, +6.1, +19 us, beside 2^24 +1.3, +5.8, +18, beside 2^26 0, 0,
-// +10. A bucket size of 2^11 then shows in 8 pairs or more up to 2^28 characters.
-constexpr uint64_t SAMPLE_MIN_N = 1ull << 24;
+// Texts at least this long are sampled (KeySample; the counting blocks take as
+// long) by as many blocks as show a bucket size of 2^11 in 8 pairs or more up to
+// 2^28 characters. Batches are sampled whatever their size: texts of few
+// letters beside texts of many hide in the batch's counts.
+constexpr uint64_t SAMPLE_MIN_N = 1ull << 22;
 // Texts of at most this many bits per character are modelled by their grams and
 // are left to them (8 characters are two digits of theirs).
 constexpr uint32_t SAMPLE_MIN_BITS = 2;
-uint32_t sample_size(uint64_t n) {
-  if (n < SAMPLE_MIN_N) return 0;
-  return n < (1ull << 25) ? 512u : n < (1ull << 27) ? 1024u : n < (1ull << 29) ? 2048u : SAMPLE_MAX;
+uint32_t sample_blocks(uint64_t n, uint32_t texts) {
+  if (n < SAMPLE_MIN_N) return texts > 1 ? 8u : 0u;
+  return n < (1ull << 26) ? 8u : n < (1ull << 28) ? 16u : SAMPLE_BLOCKS_MAX;
 }
 
-// Share of n characters in buckets of more than 2^log_large by a sample of s
-// of them that agree in `chars` characters (1 to SAMPLE_CHARS): of the bucket
-// sizes (over the characters) the agreeing pairs give the mean, the triples
-// the mean square, and a lognormal distribution with these the share; between
-// whole characters its parameters lie between theirs. Fewer than 8 pairs in
-// the whole characters or a share of 0.005 tell nothing.
-double sampled_large_share(const KeySample &k, double chars, uint32_t s, uint64_t n,
-                           double log_large) {
+// Share of n characters in buckets too large for a tile, by a sample of which
+// `pairs` and `triples` agree in `chars` characters (1 to SAMPLE_CHARS): of the
+// bucket sizes (over the characters) the pairs give the mean, the triples the
+// mean square, and a lognormal distribution has these; between whole characters
+// its parameters lie between theirs. A bucket of s items that starts anywhere
+// in a tile's window does not fit with probability (s - 512) / 2560. Fewer than
+// 8 pairs, or less than one large bucket, tell nothing.
+double sampled_large_share(const KeySample &k, double chars, uint32_t blocks, uint64_t n) {
   const uint32_t c = (uint32_t)chars;
   if (k.pairs[c - 1] < 8) return 0.0;
-  const double scale = (double)n / s;
-  auto fit = [&](uint32_t i, double &mu, double &var) {  // of the logarithm of the size
-    const double mean = 1.0 + 2.0 * std::max(0.5, (double)k.pairs[i]) / s * scale;
-    const double square = 6.0 * (double)k.triples[i] / s * scale * scale;
-    var = std::min(4.0, std::max(0.05, std::log(std::max(1.0, square / (mean * mean)))));
-    mu = std::log(mean) - var / 2;
+  const double scale = (double)n / SAMPLE_KEYS, drawn = (double)blocks * SAMPLE_KEYS;
+  auto fit = [&](uint32_t i, double &mu, double &sd) {  // of the logarithm of the size
+    const double mean = 1.0 + 2.0 * std::max(0.5, (double)k.pairs[i]) / drawn * scale;
+    const double square = 6.0 * (double)k.triples[i] / drawn * scale * scale;
+    const double var = std::log(std::max(1.0, square / (mean * mean)));
+    sd = std::sqrt(std::min(4.0, std::max(0.05, var)));
+    mu = std::log(mean) - sd * sd / 2;
   };
-  double mu, var;
-  fit(c - 1, mu, var);
+  double mu, sd;
+  fit(c - 1, mu, sd);
   if (chars > c) {
-    double mu1, var1;
-    fit(c, mu1, var1);
+    double mu1, sd1;
+    fit(c, mu1, sd1);
     mu += (chars - c) * (mu1 - mu);
-    var += (chars - c) * (var1 - var);
+    sd += (chars - c) * (sd1 - sd);
   }
-  const double z = (log_large * std::log(2.0) - mu) / std::sqrt(2.0 * var);
-  const double share = 0.5 * std::erfc(z);
-  return share < 0.005 ? 0.0 : share;
+  double share = 0, weight = 0;
+  for (double z = -3.5; z <= 3.5; z += 0.25) {  // over the normal distribution
+    const double w = std::exp(-z * z / 2);
+    share += w * std::min(1.0, std::max(0.0, (std::exp(mu + sd * z) - 512.0) / 2560.0));
+    weight += w;
+  }
+  share /= weight;
+  return share * (double)n < 1024.0 ? 0.0 : share;
 }
 
 // How the probability of a k-character prefix is spread, as the normal
@@ -368,13 +364,6 @@ struct PrefixModel {
     m.g = 8.0 / b;
     moments(p, p, RADIX, m.mean, m.var, m.least);
     moments(p, q, RADIX, m.mean1, m.var1, m.least1);
-    return m;
-  }
-
-  // `bits` of information in every character.
-  static PrefixModel uniform(double bits) {
-    PrefixModel m;
-    m.mean = m.mean1 = m.least = m.least1 = bits;
     return m;
   }
 
@@ -1487,9 +1476,14 @@ struct Build {
   // sample finds counts where it is more. Builds by the model alone and with
   // the sample: a Zipf block 4096 and 16384 times in 2^28 characters 202.8, 197.3
   // and 190.4, 186.7 ms, prose of 2^26 13.1 and 11.3, DNA beside Zipf bytes of
-  // 2^27 in all 19.6 and 17.5.
+  // 2^27 in all 19.6 and 17.5. Batches with half of every one taken to be of two
+  // bits, with the sample, unsplit: 48 texts of 10-256 KB, half DNA, half Zipf
+  // bytes 0.741, 0.743, 0.733 ms, 64 of Zipf bytes 0.525, 0.485, 0.59, 256 of
+  // protein to 1 MB 2.59, 2.17, 3.57.
   // Beyond the sample's characters its last count stands where prefixes that
-  // long are repeats (their information exceeds the length's).
+  // long are repeats (their information exceeds the length's). In a batch only
+  // whole characters of it count: a text of few letters has close codes, whose
+  // top bits divide nothing.
   uint32_t choose_split(const PrefixModel &model, const KeySample &sample, uint32_t b,
                         uint32_t segbits, uint32_t bits0) const {
     const uint32_t P = (bits0 + RADIX_BITS - 1) / RADIX_BITS;
@@ -1512,25 +1506,21 @@ struct Build {
       mass[l] = (double)chars_of[l] / (double)N;
       log_len[l] = std::log2((double)chars_of[l] / (double)texts_of[l]);
     }
-    const uint32_t sampled = S == 1 && b > SAMPLE_MIN_BITS ? sample_size(N) : 0;
+    const uint32_t sampled = b > SAMPLE_MIN_BITS ? sample_blocks(N, S) : 0;
     const bool repeats = SAMPLE_CHARS * model.mean1 >= std::log2((double)N);
-    const double few = S > 1 && b > FEW_BITS ? FEW_SHARE : 0.0;
-    const PrefixModel few_model = PrefixModel::uniform(std::min(FEW_BITS, model.mean1));
     for (uint32_t p = 1; p * RADIX_BITS < bits0; ++p) {
       const uint32_t T = p * RADIX_BITS;
       const double chars = T > segbits ? (double)(T - segbits) / b : 0.0;
       double big = 0.0, cost = p;
       for (int l = 0; l < 33; ++l)
         if (mass[l] > 0.0) {
-          const double whole = std::floor(chars);
-          big += mass[l] * ((1.0 - few) * model.large_share(chars, log_len[l], LOCAL_LARGE_LOG2) +
-                            few * few_model.large_share(whole, log_len[l], LOCAL_LARGE_LOG2));
-          cost += mass[l] * ((1.0 - few) * model.local_cost(chars, log_len[l], 8.0 / b) +
-                             few * few_model.local_cost(whole, log_len[l], 8.0 / b));
+          big += mass[l] * model.large_share(chars, log_len[l], LOCAL_LARGE_LOG2);
+          cost += mass[l] * model.local_cost(chars, log_len[l], 8.0 / b);
         }
-      if (sampled && chars >= 1.0 && (chars <= SAMPLE_CHARS || repeats))
-        big = std::max(big, sampled_large_share(sample, std::min(chars, (double)SAMPLE_CHARS), sampled,
-                                                N, LOCAL_LARGE_LOG2));
+      if (sampled && chars >= 1.0 && (chars <= SAMPLE_CHARS || repeats)) {
+        const double c = S > 1 ? std::floor(chars) : chars;
+        big = std::max(big, sampled_large_share(sample, std::min(c, (double)SAMPLE_CHARS), sampled, N));
+      }
       const uint32_t R = bits0 - T;
       if (big > 0.0) {  // its share of a pass, each with the fixed part of one
         const double rest = (R + bits_for((uint64_t)(big * N / 4096.0)) + 7) / 8;
@@ -1579,7 +1569,7 @@ struct Build {
     aa.done = &ctrl->done[0];
     aa.code = code;
     aa.seg_off = S == 1 ? segoff : nullptr;
-    aa.samples = S == 1 ? sample_size(N) : 0;
+    aa.sample_blocks = sample_blocks(N, S);
     aa.offsets = S > 1 ? segoff : nullptr;
     aa.S = S;
     if (stage_readbacks) {

@@ -10,12 +10,13 @@
 // text's critical path.
 //
 // The counts say nothing of repeats (copies of a block, words), which make
-// buckets of equal key bits large however many digits are sorted. So one more
-// block draws `samples` positions, sorts the prefixes there and counts, for 1 to
+// buckets of equal key bits large however many digits are sorted. So a few more
+// blocks each draw 512 positions, sort the prefixes there and count, for 1 to
 // SAMPLE_CHARS characters, the pairs and triples that agree in them: the mean
-// bucket size and its spread, as they are. It works beside the counting
-// blocks, on bytes, which need no codes. (1024 positions as a step of the last
-// block, on codes, took 18 us.)
+// bucket size and its spread, as they are. They work beside the counting
+// blocks, on bytes, which need no codes: +2 us beside 300 000 characters,
+// nothing from 2^22 on. (One block with 1024 positions, twice the pairs of two:
+// +11 and +7 us; as a step of the last block, on codes, +18.)
 //
 // Bound: HBM read of n bytes; 16-byte vector loads, per-warp privatised
 // shared-memory counters, one global atomic per bin and block.
@@ -27,6 +28,7 @@ namespace gbsa {
 
 constexpr int HIST_BLOCK = 512;
 constexpr int HIST_COPIES = HIST_BLOCK / 32;  // one private histogram per warp
+static_assert(SAMPLE_KEYS == HIST_BLOCK && SAMPLE_CHARS <= HIST_COPIES, "a key a thread, a warp a count");
 
 // The 8 characters at pos, first character on top, zeros from `end` on.
 __device__ __forceinline__ uint64_t prefix_at(const uint8_t *text, uint64_t n, uint64_t pos,
@@ -46,92 +48,80 @@ __device__ __forceinline__ uint64_t prefix_at(const uint8_t *text, uint64_t n, u
   return end - pos < 8 ? key & (~0ull << (8 * (8 - (end - pos)))) : key;
 }
 
-// One block: `samples` prefixes (a power of two, at least HIST_BLOCK) below
-// their text's number (textbits), sorted in `keys`.
+// One block: a prefix per thread below its text's number (textbits), sorted
+// into keys[0, SAMPLE_KEYS). `room` words of shared memory follow the keys.
 __device__ __forceinline__ void sample_prefixes(const AlphabetArgs &a, uint64_t *keys,
-                                                uint32_t textbits) {
-  const uint32_t tid = threadIdx.x, lane = tid & 31, s = a.samples;
+                                                uint32_t room, uint32_t textbits) {
+  const uint32_t tid = threadIdx.x, total = a.sample_blocks * SAMPLE_KEYS;
   const uint32_t *offsets = a.offsets;
-  if (a.S > 1 && a.S + 1 + 2 * s <= HIST_COPIES * RADIX) {  // searched in shared memory
-    uint32_t *copy = reinterpret_cast<uint32_t *>(keys + s);
+  if (a.S > 1 && a.S < room) {  // searched in shared memory
+    uint32_t *copy = reinterpret_cast<uint32_t *>(keys + SAMPLE_KEYS);
     for (uint32_t i = tid; i <= a.S; i += HIST_BLOCK) copy[i] = a.offsets[i];
     offsets = copy;
     __syncthreads();
   }
-  for (uint32_t i = tid; i < s; i += HIST_BLOCK) {
-    // Evenly spread, shifted at random: a period of the text must not show.
-    uint32_t r = i * 0x9E3779B9u;
-    r = (r ^ (r >> 16)) * 0x85EBCA6Bu;
-    r ^= r >> 13;
-    const uint64_t x = ((uint64_t)i * a.n + (((uint64_t)r * a.n) >> 32)) / s;
-    uint64_t end = a.n, text = 0;
-    if (a.S > 1) {
-      uint32_t lo = 0, hi = a.S - 1;  // the last text with an offset <= x
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (offsets[mid] <= x)
-          lo = mid;
-        else
-          hi = mid - 1;
-      }
-      end = offsets[lo + 1];
-      text = (uint64_t)lo << (64 - textbits);
+  // Evenly spread, shifted at random: a period of the text must not show.
+  const uint32_t i = tid * a.sample_blocks + blockIdx.x;
+  uint32_t r = i * 0x9E3779B9u;
+  r = (r ^ (r >> 16)) * 0x85EBCA6Bu;
+  r ^= r >> 13;
+  const uint64_t x = ((uint64_t)i * a.n + (((uint64_t)r * a.n) >> 32)) / total;
+  uint64_t end = a.n, text = 0;
+  if (a.S > 1) {
+    uint32_t lo = 0, hi = a.S - 1;  // the last text with an offset <= x
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (offsets[mid] <= x)
+        lo = mid;
+      else
+        hi = mid - 1;
     }
-    keys[i] = text | (prefix_at(a.text, a.n, x, end) >> textbits);
+    end = offsets[lo + 1];
+    text = (uint64_t)lo << (64 - textbits);
+  }
+  uint64_t key = text | (prefix_at(a.text, a.n, x, end) >> textbits);
+  // Bitonic: steps inside a warp by shuffles, the others in shared memory.
+  for (uint32_t k = 2; k <= SAMPLE_KEYS; k <<= 1) {
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      uint64_t q;
+      if (j >= 32) {
+        __syncthreads();  // the step before is read
+        keys[tid] = key;
+        __syncthreads();
+        q = keys[tid ^ j];
+      } else {
+        q = __shfl_xor_sync(0xffffffffu, key, j);
+      }
+      const bool least = ((tid & j) == 0) == ((tid & k) == 0);
+      key = (q < key) == least ? q : key;
+    }
   }
   __syncthreads();
-  // Bitonic; the steps inside rows of 32 by shuffles.
-  for (uint32_t k0 = 32; k0 <= s; k0 <<= 1) {
-    for (uint32_t j = k0 >> 1; j >= 32; j >>= 1) {
-      for (uint32_t i = tid; i < s / 2; i += HIST_BLOCK) {
-        const uint32_t lo = 2 * i - (i & (j - 1)), hi = lo + j;
-        const uint64_t p = keys[lo], q = keys[hi];
-        if ((p > q) == ((lo & k0) == 0)) {
-          keys[lo] = q;
-          keys[hi] = p;
-        }
-      }
-      __syncthreads();
-    }
-    for (uint32_t i = tid; i < s; i += HIST_BLOCK) {
-      uint64_t p = keys[i];
-      for (uint32_t k = k0 == 32 ? 2 : k0; k <= k0; k <<= 1) {
-        for (uint32_t j = min(k >> 1, 16u); j > 0; j >>= 1) {
-          const uint64_t q = __shfl_xor_sync(0xffffffffu, p, j);
-          const bool least = ((lane & j) == 0) == ((i & k) == 0);
-          p = (q < p) == least ? q : p;
-        }
-      }
-      keys[i] = p;
-    }
-    __syncthreads();
-  }
+  keys[tid] = key;
+  __syncthreads();
 }
 
-// One warp: the pairs and triples of the sorted keys that agree in their top
-// `bits`. A key agrees with every one from its group's head on.
-__device__ __forceinline__ void count_agreeing(const uint64_t *keys, uint32_t s, uint32_t bits,
-                                               uint32_t *pairs_out, unsigned long long *triples_out) {
+// One warp: adds the pairs and triples of the sorted keys that agree in their
+// top `bits`. A key agrees with every one from its group's head on.
+__device__ __forceinline__ void count_agreeing(const uint64_t *keys, uint32_t bits, uint32_t *pairs,
+                                               unsigned long long *triples) {
   const uint32_t lane = threadIdx.x & 31, R = 64 - bits;
-  uint32_t first = 0;  // the last head so far
-  unsigned long long pairs = 0, triples = 0;
-  for (uint32_t i0 = 0; i0 < s; i0 += 32) {
+  uint32_t first = 0, p = 0, t = 0;  // the last head so far; p, t below 2^32 in all
+#pragma unroll 4
+  for (uint32_t i0 = 0; i0 < SAMPLE_KEYS; i0 += 32) {
     const uint32_t i = i0 + lane;
     const bool head = i == 0 || ((keys[i] ^ keys[i - 1]) >> R) != 0;
     const uint32_t H = __ballot_sync(0xffffffffu, head), m = H & (lanemask_lt() | (1u << lane));
-    const unsigned long long before = i - (m ? i0 + 31 - __clz(m) : first);
-    pairs += before;
-    triples += before * (before - 1) / 2;
+    const uint32_t before = i - (m ? i0 + 31 - __clz(m) : first);
+    p += before;
+    t += before * (before - 1) / 2;
     if (H) first = i0 + 31 - __clz(H);
   }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    pairs += __shfl_xor_sync(0xffffffffu, pairs, d);
-    triples += __shfl_xor_sync(0xffffffffu, triples, d);
-  }
+  p = __reduce_add_sync(0xffffffffu, p);
+  t = __reduce_add_sync(0xffffffffu, t);
   if (lane == 0) {
-    *pairs_out = (uint32_t)pairs;
-    *triples_out = triples;
+    atomicAdd(pairs, p);
+    atomicAdd(triples, (unsigned long long)t);
   }
 }
 
@@ -173,21 +163,18 @@ __device__ __forceinline__ void count_bytes(const AlphabetArgs &a, uint32_t (*s_
 }
 
 __global__ void __launch_bounds__(HIST_BLOCK, 4) k_byte_histogram(AlphabetArgs a) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
+  __shared__ __align__(16) uint32_t s_hist[HIST_COPIES][RADIX];
   uint32_t *hist = a.hist;
   const uint64_t n = a.n;
-  const uint32_t sampling = a.samples ? 1u : 0u;
-  if (blockIdx.x < sampling) {
-    uint64_t *keys = reinterpret_cast<uint64_t *>(smem_raw);
+  if (blockIdx.x < a.sample_blocks) {
+    uint64_t *keys = reinterpret_cast<uint64_t *>(s_hist);
     const uint32_t textbits = a.S > 1 ? 32 - __clz(a.S - 1) : 0;
-    sample_prefixes(a, keys, textbits);
+    sample_prefixes(a, keys, HIST_COPIES * RADIX - 2 * SAMPLE_KEYS, textbits);
     KeySample *out = reinterpret_cast<KeySample *>(hist + RADIX);
     const uint32_t w = threadIdx.x >> 5, bits = textbits + 8 * (w + 1);
-    if (w < SAMPLE_CHARS && bits <= 64)
-      count_agreeing(keys, a.samples, bits, &out->pairs[w], &out->triples[w]);
+    if (w < SAMPLE_CHARS && bits <= 64) count_agreeing(keys, bits, &out->pairs[w], &out->triples[w]);
   } else {
-    count_bytes(a, reinterpret_cast<uint32_t (*)[RADIX]>(smem_raw), blockIdx.x - sampling,
-                gridDim.x - sampling);
+    count_bytes(a, s_hist, blockIdx.x - a.sample_blocks, gridDim.x - a.sample_blocks);
   }
   __shared__ uint32_t s_last, s_tmp[HIST_COPIES + 1];
   __syncthreads();
@@ -214,10 +201,10 @@ __global__ void __launch_bounds__(HIST_BLOCK, 4) k_byte_histogram(AlphabetArgs a
 cudaError_t launch_byte_histogram(const AlphabetArgs &a, int num_sms, cudaStream_t stream) {
   if (a.n == 0) return cudaSuccess;
   uint64_t want = (a.n / 16 + HIST_BLOCK - 1) / HIST_BLOCK;
-  uint64_t cap = (uint64_t)num_sms * 4 - (a.samples ? 1 : 0);  // resident at once
+  if (a.sample_blocks > SAMPLE_BLOCKS_MAX) return cudaErrorInvalidValue;
+  uint64_t cap = std::max<uint64_t>(1, (uint64_t)num_sms * 4 - a.sample_blocks);  // all resident
   unsigned grid = (unsigned)(want < 1 ? 1 : (want > cap ? cap : want));
-  const size_t smem = std::max<size_t>(HIST_COPIES * RADIX * 4, (size_t)a.samples * 8);
-  k_byte_histogram<<<grid + (a.samples ? 1 : 0), HIST_BLOCK, smem, stream>>>(a);
+  k_byte_histogram<<<grid + a.sample_blocks, HIST_BLOCK, 0, stream>>>(a);
   return cudaGetLastError();
 }
 

@@ -36,9 +36,9 @@ cudaError_t launch_copy_words(uint32_t *dst, const uint32_t *src, uint64_t words
 cudaError_t launch_copy_bytes(uint8_t *dst, const uint8_t *src, uint64_t n, cudaStream_t stream);
 
 // ---- step A0: alphabet (k_alphabet.cu) ----------------------------------
-// Of `samples` prefixes: pairs and triples of one text that agree in 1, 2, ..
-// characters (0 beyond what 64 bits hold beside the text's number).
-constexpr uint32_t SAMPLE_MAX = 4096, SAMPLE_CHARS = 8;
+// Of the prefixes drawn: pairs and triples of one block and text that agree in
+// 1, 2, .. characters (0 beyond what 64 bits hold beside the text's number).
+constexpr uint32_t SAMPLE_KEYS = 512, SAMPLE_CHARS = 8, SAMPLE_BLOCKS_MAX = 64;
 struct KeySample {
   unsigned long long triples[SAMPLE_CHARS];
   uint32_t pairs[SAMPLE_CHARS];
@@ -51,7 +51,7 @@ struct AlphabetArgs {
   uint8_t *code;      // out: dense order-preserving code of each byte value
   uint32_t *seg_off;  // out, for one text: {0, n} (NULL otherwise)
   uint32_t *host;     // out: the counts and the sample in pinned host memory, or NULL
-  uint32_t samples;   // prefixes to draw: 0 or a power of two in [512, SAMPLE_MAX]
+  uint32_t sample_blocks;  // blocks that draw SAMPLE_KEYS prefixes each (0: none)
   const uint32_t *offsets;  // S + 1 offsets of a batch (S > 1)
   uint32_t S;
   uint32_t *host_flag;  // set to 1 after them

@@ -32,7 +32,7 @@ def copies(n, count, seed):
     return t
 
 
-N = (1 << 24) + 77  # the shortest texts that are sampled, and a few more
+N = (1 << 22) + 77  # the shortest texts that are sampled, and a few more
 
 
 @pytest.mark.parametrize("make,split", [(lambda: gen.text("zipf", 3, N), True), (lambda: gen.text("bytes", 4, N), True),
@@ -57,3 +57,35 @@ def test_sampled_alphabets_and_alignments(gb, orc, symbols, offset):
     d = torch.empty(N + 16, dtype=torch.uint8, device="cuda")[offset:offset + N]
     d.copy_(torch.from_numpy(t))
     assert orc.check_sa(t, u32(gb.sa_build(d))) == (0, -1)
+
+
+def test_batches_are_measured(gb, orc):
+    """Texts of four letters beside texts of many need more digits than either
+    the batch's counts or a batch of like texts."""
+    import torch
+    size, count, passes = 60001, 24, {}
+    for kinds in (("zipf", "zipf"), ("protein", "protein"), ("zipf", "dna")):
+        rng = np.random.default_rng(9)
+        texts = [rng.integers(0, 20, size - 11 * k).astype(np.uint8) if kinds[k % 2] == "protein" else
+                 gen.text(kinds[k % 2], 70 + k, size - 11 * k) for k in range(count)]
+        off = np.concatenate([[0], np.cumsum([x.size for x in texts])]).astype(np.uint64)
+        sa, st = gb.sa_build_batched(torch.from_numpy(np.concatenate(texts)).cuda(), off, stats=True)
+        got = u32(sa)
+        for k, x in enumerate(texts):
+            assert np.array_equal(got[int(off[k]):int(off[k + 1])], orc.pd_sa(x)[0]), k
+        passes[kinds[1]] = st["passes"][0]
+    assert passes["protein"] < passes["zipf"] < passes["dna"]
+
+
+@pytest.mark.parametrize("count,size", [(2, 3), (2, 5000), (700, 90), (3571, 40), (3572, 40), (9000, 7)])
+def test_sampled_batches(gb, orc, count, size):
+    """Batches whose offsets the sample holds in shared memory, and larger ones."""
+    import torch
+    rng = np.random.default_rng(count)
+    texts = [rng.integers(0, 40, int(rng.integers(0, size + 1))).astype(np.uint8) for _ in range(count)]
+    texts[0] = np.arange(3, dtype=np.uint8)
+    off = np.concatenate([[0], np.cumsum([x.size for x in texts])]).astype(np.uint64)
+    got = u32(gb.sa_build_batched(torch.from_numpy(np.concatenate(texts)).cuda(), off))
+    for k in range(0, count, 1 + count // 300):
+        if texts[k].size:
+            assert np.array_equal(got[int(off[k]):int(off[k + 1])], orc.pd_sa(texts[k])[0]), k
