@@ -465,7 +465,7 @@ struct Build {
   // Launches whose byte counts wait for the round's control block.
   static constexpr uint64_t PENDING = ~0ull;
   struct Pending {
-    uint32_t scatter = 0, apply = 0, bucket_upd = 0, bucket_surv = 0;
+    uint32_t scatter = 0, apply = 0, bucket_upd = 0, bucket_surv = 0, classify = 0;
   } pend;
   std::vector<cudaEvent_t> evpool;
   size_t evused = 0;
@@ -748,7 +748,7 @@ struct Build {
   }
 
   // Large groups and the refine tile map of the list just written.
-  sa_status classify(int out, uint64_t cap_groups, uint32_t apply_bound) {
+  sa_status classify(int out, uint32_t apply_bound) {
     ClassifyArgs ca{};
     ca.gstart = gstart[out];
     ca.gname = gname[out];
@@ -766,7 +766,8 @@ struct Build {
     ca.max_groups = L.max_groups;
     ca.max_tiles = L.max_tiles;
     ca.ctrl = ctrl;
-    sa_status s = launch(SA_K_CLASSIFY, 0, 16 * cap_groups,
+    ++pend.classify;
+    sa_status s = launch(SA_K_CLASSIFY, 0, PENDING,
                          [&] { return launch_classify(ca, sm_count(), st); });
     if (s != SA_OK) return s;
     // ISA entries of the rename's survivors whose name changed, bucketed by
@@ -843,17 +844,29 @@ struct Build {
   // entry; bucketing reads 8 (histogram), then reads and writes 8.
   void settle(const HostCtrl &hc) {
     bytes += pend.scatter * 12ull * hc.upd + pend.apply * 12ull * hc.m_l +
-             pend.bucket_upd * 24ull * hc.upd + pend.bucket_surv * 24ull * hc.m_l;
+             pend.bucket_upd * 24ull * hc.upd + pend.bucket_surv * 24ull * hc.m_l +
+             pend.classify * classify_bytes(hc);
     pend = Pending{};
     for (Rec &r : recs) {
       if (r.bytes != PENDING) continue;
       if (r.cls == SA_K_SCATTER) r.bytes = 12ull * hc.upd;
       if (r.cls == SA_K_APPLY) r.bytes = 12ull * hc.m_l;
+      if (r.cls == SA_K_CLASSIFY) r.bytes = classify_bytes(hc);
       if (r.cls == SA_K_BUCKET && (r.pass & 4))
         r.bytes = 0;
       else if (r.cls == SA_K_BUCKET)
         r.bytes = ((r.pass & 1) ? 16ull : 8ull) * ((r.pass & 2) ? hc.m_l : hc.upd);
     }
+  }
+
+  // Classification: 4 bytes (start) per group, 12 (head rank, parent's name,
+  // name) per group that the rename wrote, 4 per refine tile, 20 (head rank
+  // and the four lists) per large group.
+  uint64_t classify_bytes(uint32_t items, uint32_t groups, uint32_t renamed, uint32_t large) const {
+    return 4ull * groups + 12ull * renamed + 4ull * (items / nominal + 1) + 20ull * large;
+  }
+  uint64_t classify_bytes(const HostCtrl &hc) const {
+    return classify_bytes(hc.m_next(), hc.g_next(), hc.g_l, hc.g_large());
   }
 
   // Rename (round 0 or large groups) reads 12 bytes per item; writes 4 (SA)
@@ -1198,8 +1211,9 @@ struct Build {
       const uint32_t kbits = x.mL ? W + (x.GL > 1 ? bits_for(x.GL - 1) : 0) : 0;
       const uint64_t rbl = x.mL ? rename_bytes(x.mL, x.m_l, x.g_l) : 0;
       const uint64_t rfb = refine_bytes(x.m - x.mL, x.G - x.GL, x.m_s, x.g_s, x.upd, 2);
-      bytes += (x.mL ? (uint64_t)x.passes * 24 * x.mL + 32ull * x.mL : 0) + rbl + rfb + 8ull * x.G +
-               12ull * x.upd + (x.m >= bucket_min ? 24ull * x.upd : 0) +
+      const uint32_t next_large = r < last ? rec[r + 1].GL : 0;
+      bytes += (x.mL ? (uint64_t)x.passes * 24 * x.mL + 32ull * x.mL : 0) + rbl + rfb +
+               classify_bytes(x.m_s + x.m_l, x.g_s + x.g_l, x.g_l, next_large) + 12ull * x.upd + (x.m >= bucket_min ? 24ull * x.upd : 0) +
                (x.mL ? 12ull * x.m_l + (x.mL >= bucket_min ? 24ull * x.m_l : 0) : 0);
       launches += 5 + (x.mL ? 12 + MAX_PASSES - 1 : 0) + (x.m >= bucket_min ? 3 : 0) +
                   (x.mL && x.mL >= bucket_min ? 3 : 0);
@@ -1245,13 +1259,13 @@ struct Build {
     small = nominal = half;
     if (!again) return SA_OK;
     CK(cudaMemsetAsync(&ctrl->rc.large, 0, sizeof(ctrl->rc.large), st));
-    sa_status s = classify(cur, hc.g_next(), 0);
+    sa_status s = classify(cur, 0);
     if (s != SA_OK) return s;
     HostCtrl h2{};
     s = read_ctrl(h2);
     if (s != SA_OK) return s;
     hc.large = h2.large;
-    bytes += 8ull * hc.g_next();
+    settle(h2);
     return flush(0, 0);
   }
 
@@ -1290,14 +1304,14 @@ struct Build {
     if (s != SA_OK) return s;
     launches += 3;
     bytes += rank_bytes + move_bytes;
-    s = classify(nxt, G, 0);
+    s = classify(nxt, 0);
     if (s != SA_OK) return s;
     HostCtrl h2{};
     s = read_ctrl(h2);
     if (s != SA_OK) return s;
+    settle(h2);
     s = flush(0, 0);
     if (s != SA_OK) return s;
-    bytes += 8ull * G;
     h2.passes = hc.passes;
     h2.pass_mask = hc.pass_mask;
     h2.upd = hc.upd;
@@ -1398,8 +1412,7 @@ struct Build {
     s = clear_isa();
     if (s != SA_OK) return s;
     CK(cudaMemsetAsync(&ctrl->rc.large, 0, sizeof(ctrl->rc.large), st));
-    const uint32_t g_cap = hc.g_s + mL / 2 + 1;
-    s = classify(out, g_cap, mL);
+    s = classify(out, mL);
     if (s != SA_OK) return s;
     s = read_ctrl(hc);
     if (s != SA_OK) return s;
@@ -1407,7 +1420,7 @@ struct Build {
     settle(hc);
     s = flush(hc.pass_mask, rb);
     if (s != SA_OK) return s;
-    bytes += (mL ? (uint64_t)hc.passes * 24 * mL : 0) + rb + 8ull * g_cap;
+    bytes += (mL ? (uint64_t)hc.passes * 24 * mL : 0) + rb;
     hc.passes = passes + (mL ? hc.passes : 0);
     return SA_OK;
   }
@@ -1699,7 +1712,7 @@ struct Build {
       if (s != SA_OK) return s;
       s = rename(N32, 1, cb, c0, 0, nullptr, nullptr, 0, cur, ctrl->zero);
       if (s != SA_OK) return s;
-      s = classify(cur, N / 2 + 1, N32);
+      s = classify(cur, N32);
       if (s != SA_OK) return s;
       s = read_ctrl(hc);
       if (s != SA_OK) return s;
@@ -1870,7 +1883,7 @@ struct Build {
       }
       s = scatter(m);
       if (s != SA_OK) return s;
-      s = classify(nxt, G, mL);
+      s = classify(nxt, mL);
       if (s != SA_OK) return s;
       if (opt.trace_isa && round < opt.trace_cap && S == 1)
         CK(cudaMemcpyAsync(opt.trace_isa + (size_t)round * N, isa, N * 4,
@@ -1889,7 +1902,7 @@ struct Build {
       s = flush(hc.pass_mask, rbl, p1[1]);
       if (s != SA_OK) return s;
       record(round, m, hc, kbits);
-      bytes += (mL ? (uint64_t)hc.passes * 24 * mL : 0) + rbl + rfb + 8ull * G;
+      bytes += (mL ? (uint64_t)hc.passes * 24 * mL : 0) + rbl + rfb;
       cur = nxt;
       h *= mult;
       ++round;
