@@ -2,8 +2,13 @@
 // inverse-suffix-array form (Section 2.1, Algorithms 1, 4 and 5).
 //
 // Round 0 (initial names, Algorithm 1's first lines):
-//   byte histogram -> alphabet (host) -> packed keys -> radix sort ->
-//   rename/unique/compact.
+//   byte histogram and a sample of prefixes -> alphabet and number of digits
+//   (host, choose_split) -> packed keys -> radix sort of the top digits ->
+//   sort/rename/unique/compact of the buckets of equal top bits tile by tile
+//   (k_local.cu; buckets too large for a tile: radix sort of their other
+//   digits and k_rename), or radix sort of all digits -> k_rename; then the
+//   ISA entries of the suffixes already final that later rounds read
+//   (k_isa.cu) and, in large texts, the groups in position order (k_reorder.cu).
 // Round r >= 1 (one doubling step, h = c0 * 2^(r-1) characters resolved):
 //   large groups: partner-name gather -> radix sort of (group, partner)
 //   keys; small groups: tile-local refine (k_refine.cu); then the rename of
@@ -19,7 +24,9 @@
 //
 // Host <-> device per round: one 64-byte read of the control block (active
 // and group counts of both producers, large-group counts, pass count, error
-// word) at the end of the round.
+// word) at the end of the round. Round 0 reads the byte counts and the sample
+// first and, from buckets, the control block before and after the large ones'
+// rename; reports that a kernel writes to pinned memory are polled.
 //
 // Data layout in HBM (N characters in S texts, gapped positions N + S):
 //   keys A/B u64[N], vals A/B u32[N] (radix sort of round 0 and of large
@@ -254,12 +261,16 @@ constexpr double RENAME_COST = 1.5;
 constexpr double PASS_FIXED_US = 9.0, PASS_ITEM_US = 7e-6;
 constexpr uint32_t REFINE_HALF_MIN = 1u << 19;
 constexpr uint64_t LOCAL_REPORT_MAX = 1ull << 22;
-// log2 of the bucket size that a tile takes about half of the time: buckets
-// of up to 512 items always fit, of 3072 and more never.
+// log2 of the bucket size from which the model takes buckets to be too large
+// for a tile. A tile takes one of s items with probability (3072 - s) / 2560,
+// half of those of 2^10.8 and 71 % here. With 10.8 the choices for Zipf bytes,
+// protein and random bytes of 2^20 to 2^30 characters are the same, but for two
+// digits instead of three for random bytes of 2^26: 3.71 ms, 2.57.
 constexpr double LOCAL_LARGE_LOG2 = 10.3;
-// From this length on, with at most a quarter of the suffixes active, the ISA gets only the entries that later rounds read
-// (k_isa.cu), and from the second on they go through a list that can be
-// bucketed by position (an ISA that the L2 holds is written directly).
+// From the first length on, with at most a quarter of the suffixes active,
+// the ISA gets only the entries that later rounds read (k_isa.cu), and from
+// the second on they go through a list that can be bucketed by position (an
+// ISA that the L2 holds is written directly).
 constexpr uint64_t NEED_MIN_N = 1ull << 22, COLLECT_MIN_N = 1ull << 25;
 // Texts at least this long wait for the gram histogram to model their
 // prefixes by its statistics; shorter ones take the character counts.
@@ -1126,9 +1137,9 @@ struct Build {
     rs0.h_next = h1;
     rs0.epoch = epoch + ROUND_EPOCHS;
     CK(cudaMemcpyAsync(&ctrl->rs, &rs0, sizeof(rs0), cudaMemcpyHostToDevice, st));
-    // Round 0's kernels already set the attributes of the sort and rename
-    // kernels; the refine's are set when it is first captured (a host call
-    // that capture allows).
+    // Kernels that round 0 did not launch (the refine, and the rename where the
+    // buckets took its place) set their attributes when first captured, a host
+    // call that capture allows.
     cudaStream_t cs = nullptr, cs2 = nullptr;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1213,7 +1224,8 @@ struct Build {
       const uint64_t rfb = refine_bytes(x.m - x.mL, x.G - x.GL, x.m_s, x.g_s, x.upd, 2);
       const uint32_t next_large = r < last ? rec[r + 1].GL : 0;
       bytes += (x.mL ? (uint64_t)x.passes * 24 * x.mL + 32ull * x.mL : 0) + rbl + rfb +
-               classify_bytes(x.m_s + x.m_l, x.g_s + x.g_l, x.g_l, next_large) + 12ull * x.upd + (x.m >= bucket_min ? 24ull * x.upd : 0) +
+               classify_bytes(x.m_s + x.m_l, x.g_s + x.g_l, x.g_l, next_large) +
+               12ull * x.upd + (x.m >= bucket_min ? 24ull * x.upd : 0) +
                (x.mL ? 12ull * x.m_l + (x.mL >= bucket_min ? 24ull * x.m_l : 0) : 0);
       launches += 5 + (x.mL ? 12 + MAX_PASSES - 1 : 0) + (x.m >= bucket_min ? 3 : 0) +
                   (x.mL && x.mL >= bucket_min ? 3 : 0);
@@ -1506,9 +1518,6 @@ struct Build {
   uint32_t choose_split(const PrefixModel &model, const KeySample &sample, uint32_t b,
                         uint32_t segbits, uint32_t bits0) const {
     const uint32_t P = (bits0 + RADIX_BITS - 1) / RADIX_BITS;
-#ifdef GBSA_SPLIT_PASSES
-    return std::min<uint32_t>(GBSA_SPLIT_PASSES, (bits0 - 1) / RADIX_BITS);
-#endif
     double best = P + RENAME_COST;
     uint32_t split = 0;
     // Characters by the logarithm of their text's length.
@@ -1543,7 +1552,8 @@ struct Build {
       const uint32_t R = bits0 - T;
       if (big > 0.0) {  // its share of a pass, each with the fixed part of one
         const double rest = (R + bits_for((uint64_t)(big * N / 4096.0)) + 7) / 8;
-        const double share = (big * N * PASS_ITEM_US + PASS_FIXED_US) / (N * PASS_ITEM_US + PASS_FIXED_US);
+        const double share =
+            (big * N * PASS_ITEM_US + PASS_FIXED_US) / (N * PASS_ITEM_US + PASS_FIXED_US);
         cost += share * (rest + 3.0 + RENAME_COST);
       }
       if (cost < best) {

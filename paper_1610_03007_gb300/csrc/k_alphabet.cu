@@ -28,7 +28,8 @@ namespace gbsa {
 
 constexpr int HIST_BLOCK = 512;
 constexpr int HIST_COPIES = HIST_BLOCK / 32;  // one private histogram per warp
-static_assert(SAMPLE_KEYS == HIST_BLOCK && SAMPLE_CHARS <= HIST_COPIES, "a key a thread, a warp a count");
+static_assert(SAMPLE_KEYS == HIST_BLOCK && SAMPLE_CHARS <= HIST_COPIES,
+              "a key to a thread, a count to a warp");
 
 // The 8 characters at pos, first character on top, zeros from `end` on.
 __device__ __forceinline__ uint64_t prefix_at(const uint8_t *text, uint64_t n, uint64_t pos,
