@@ -320,8 +320,9 @@ double sampled_large_share(const KeySample &k, double chars, uint32_t blocks, ui
     mu += (chars - c) * (mu1 - mu);
     sd += (chars - c) * (sd1 - sd);
   }
+  if (mu + 3.5 * sd <= std::log(512.0)) return 0.0;
   double share = 0, weight = 0;
-  for (double z = -3.5; z <= 3.5; z += 0.25) {  // over the normal distribution
+  for (double z = -3.5; z <= 3.5; z += 0.5) {  // over the normal distribution
     const double w = std::exp(-z * z / 2);
     share += w * std::min(1.0, std::max(0.0, (std::exp(mu + sd * z) - 512.0) / 2560.0));
     weight += w;
@@ -1549,6 +1550,7 @@ struct Build {
           big += mass[l] * model.large_share(chars, log_len[l], LOCAL_LARGE_LOG2);
           cost += mass[l] * model.local_cost(chars, log_len[l], 8.0 / b);
         }
+      if (cost >= best) continue;
       if (sampled && chars >= 1.0 && (chars <= SAMPLE_CHARS || repeats)) {
         const double c = S > 1 ? std::floor(chars) : chars;
         const double found =
