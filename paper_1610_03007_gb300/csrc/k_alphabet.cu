@@ -188,13 +188,15 @@ __global__ void __launch_bounds__(HIST_BLOCK, 4) k_byte_histogram(AlphabetArgs a
   __threadfence();
   const uint32_t d = threadIdx.x;
   const uint32_t c = d < RADIX ? load_volatile_u32(hist + d) : 0u;
+  const bool sampled = a.sample_blocks && a.host && d < sizeof(KeySample) / 4;
+  const uint32_t w = sampled ? load_volatile_u32(hist + RADIX + d) : 0u;
   uint32_t sigma;
   const uint32_t code = block_exclusive<HIST_BLOCK>(c ? 1u : 0u, OpAdd(), 0u, s_tmp, sigma);
   if (d < RADIX) {
     a.code[d] = (uint8_t)code;
     if (a.host) a.host[d] = c;
   }
-  if (a.host && d < sizeof(KeySample) / 4) a.host[RADIX + d] = load_volatile_u32(hist + RADIX + d);
+  if (sampled) a.host[RADIX + d] = w;
   if (d < 2 && a.seg_off) a.seg_off[d] = d ? (uint32_t)n : 0u;
   if (a.host) report_to_host(a.host_flag);
 }
