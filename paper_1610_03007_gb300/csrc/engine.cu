@@ -1445,8 +1445,9 @@ struct Build {
   }
 
   // ISA entries of the final ranks in the SA: all, or those whose position
-  // is in `missing`. The list goes through the active buffer `buf`.
-  sa_status collect(int buf, const uint32_t *missing) {
+  // is in `missing`, into out[0, len). The list goes through the active
+  // buffer `buf`.
+  sa_status collect(int buf, const uint32_t *missing, uint32_t *out, uint64_t len) {
     CollectArgs ca{};
     ca.sa = sa;
     ca.N = (uint32_t)N;
@@ -1472,7 +1473,7 @@ struct Build {
     s = next_launch(ctr, ep);
     if (s != SA_OK) return s;
     return launch(SA_K_SCATTER, 3, 0, [&] {
-      return launch_write_entries(src, &ctrl->need_entries, (uint32_t)N, isa, N + S + 1, ctr,
+      return launch_write_entries(src, &ctrl->need_entries, (uint32_t)N, out, len, ctr,
                                   8 * sm_count(), st);
     });
   }
@@ -1501,7 +1502,7 @@ struct Build {
     if (s != SA_OK) return s;
     ++launches;
     bytes += 8ull * m;
-    return collect(from ^ 1, na.missing);
+    return collect(from ^ 1, na.missing, isa, N + S + 1);
   }
 
   // Digits of the top that the radix sort of round 0 takes before the
@@ -1752,8 +1753,13 @@ struct Build {
     bytes -= keys_in_pass ? 11ull * m : 0ull;
     // The unique suffixes' ISA entries are needed only by a later round, the
     // ISA output or the trace; a text resolved in round 0 skips them.
+    // Without a later round or the trace the ISA output needs no array of its
+    // own to be copied from (one text: gapped positions are its own).
+    const bool direct = isa_out && hc.m_next() == 0 && !want_trace;
+    uint32_t *const fill = direct ? isa_out : isa;
+    const uint64_t fill_len = direct ? N : N + S + 1;
     if (hc.m_next() > 0 || isa_out || want_trace) {
-      s = clear_isa();
+      if (!direct) s = clear_isa();
       if (s != SA_OK) return s;
       need_filtered = !isa_out && !opt.trace_isa && !device_rounds_wanted() && N >= NEED_MIN_N &&
                       hc.m_next() <= N / 4;
@@ -1763,10 +1769,10 @@ struct Build {
       } else if (N < COLLECT_MIN_N || bucket_min == 0xFFFFFFFFu) {
         bytes += 8ull * N;
         s = launch(SA_K_SCATTER, 1, 8ull * N, [&] {
-          return launch_isa_fill(sa, N32, segoff, S, isa, N + S + 1, st);
+          return launch_isa_fill(sa, N32, segoff, S, fill, fill_len, st);
         });
       } else {
-        s = collect(cur ^ 1, nullptr);
+        s = collect(cur ^ 1, nullptr, fill, fill_len);
       }
       if (s != SA_OK) return s;
       // Its records settle with round 0's counts, before round 1 reads new ones.
@@ -1931,7 +1937,7 @@ struct Build {
       ++round;
     }
     // ---- output ----
-    if (isa_out) {
+    if (isa_out && !direct) {
       s = launch(SA_K_OUTPUT, 0, 8ull * N, [&] {
         return launch_isa_to_local(isa, isa_out, N32, segoff, S, st);
       });

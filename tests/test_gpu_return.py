@@ -23,7 +23,9 @@ def u32(x):
 
 
 @pytest.mark.parametrize("recipe,n,kw", [("dna", 1, {"isa": True}), ("dna", 1 << 24, {"isa": True}),
-                                         ("zipf_repeats", 1 << 22, {"isa": True}),
+                                         ("zipf_repeats", 1 << 22, {"isa": True}), ("dna", (1 << 25) + 3, {"isa": True}),
+                                         ("dna", (1 << 25) + 3, {"isa": True, "bucket_min": 1 << 20}),
+                                         ("dna", 70001, {"isa": True, "trace_cap": 2}),
                                          ("dna", 1 << 24, {"trace_cap": 1})])
 def test_nothing_left_on_the_stream(gb, orc, recipe, n, kw):
     import torch
