@@ -28,6 +28,9 @@ namespace gbsa {
 
 constexpr int HIST_BLOCK = 512;
 constexpr int HIST_COPIES = HIST_BLOCK / 32;  // one private histogram per warp
+// Texts of at most this many characters (two bits) are modelled by their grams:
+// a block that meets no more stops (5 us of a batch of DNA).
+constexpr int SAMPLE_MIN_SIGMA = 4;
 static_assert(SAMPLE_KEYS == HIST_BLOCK && SAMPLE_CHARS <= HIST_COPIES,
               "a key to a thread, a count to a warp");
 
@@ -50,8 +53,9 @@ __device__ __forceinline__ uint64_t prefix_at(const uint8_t *text, uint64_t n, u
 }
 
 // One block: a prefix per thread below its text's number (textbits), sorted
-// into keys[0, SAMPLE_KEYS). `room` words of shared memory follow the keys.
-__device__ __forceinline__ void sample_prefixes(const AlphabetArgs &a, uint64_t *keys,
+// into keys[0, SAMPLE_KEYS); false, and none, when they start with at most
+// SAMPLE_MIN_SIGMA characters. `room` words of shared memory follow the keys.
+__device__ __forceinline__ bool sample_prefixes(const AlphabetArgs &a, uint64_t *keys,
                                                 uint32_t room, uint32_t textbits) {
   const uint32_t tid = threadIdx.x, total = a.sample_blocks * SAMPLE_KEYS;
   const uint32_t *offsets = a.offsets;
@@ -80,7 +84,21 @@ __device__ __forceinline__ void sample_prefixes(const AlphabetArgs &a, uint64_t 
     end = offsets[lo + 1];
     text = (uint64_t)lo << (64 - textbits);
   }
-  uint64_t key = text | (prefix_at(a.text, a.n, x, end) >> textbits);
+  const uint64_t prefix = prefix_at(a.text, a.n, x, end);
+  uint64_t key = text | (prefix >> textbits);
+  // The characters that start a prefix: a set of 256 bits.
+  __shared__ uint32_t s_seen[RADIX / 32];
+  if (tid < RADIX / 32) s_seen[tid] = 0u;
+  __syncthreads();
+  const uint32_t c = (uint32_t)(prefix >> 56);
+  for (uint32_t w = 0; w < RADIX / 32; ++w) {
+    const uint32_t in = __reduce_or_sync(0xffffffffu, c / 32 == w ? 1u << (c & 31) : 0u);
+    if ((tid & 31) == 0 && in) atomicOr(&s_seen[w], in);
+  }
+  __syncthreads();
+  int seen = 0;
+  for (uint32_t w = 0; w < RADIX / 32; ++w) seen += __popc(s_seen[w]);
+  if (seen <= SAMPLE_MIN_SIGMA) return false;  // the same for every thread
   // Bitonic: steps inside a warp by shuffles, the others in shared memory.
   for (uint32_t k = 2; k <= SAMPLE_KEYS; k <<= 1) {
     for (uint32_t j = k >> 1; j > 0; j >>= 1) {
@@ -100,6 +118,7 @@ __device__ __forceinline__ void sample_prefixes(const AlphabetArgs &a, uint64_t 
   __syncthreads();
   keys[tid] = key;
   __syncthreads();
+  return true;
 }
 
 // One warp: adds the pairs and triples of the sorted keys that agree in their
@@ -170,10 +189,11 @@ __global__ void __launch_bounds__(HIST_BLOCK, 4) k_byte_histogram(AlphabetArgs a
   if (blockIdx.x < a.sample_blocks) {
     uint64_t *keys = reinterpret_cast<uint64_t *>(s_hist);
     const uint32_t textbits = a.S > 1 ? 32 - __clz(a.S - 1) : 0;
-    sample_prefixes(a, keys, HIST_COPIES * RADIX - 2 * SAMPLE_KEYS, textbits);
+    const bool taken = sample_prefixes(a, keys, HIST_COPIES * RADIX - 2 * SAMPLE_KEYS, textbits);
     KeySample *out = reinterpret_cast<KeySample *>(hist + RADIX);
     const uint32_t w = threadIdx.x >> 5, bits = textbits + 8 * (w + 1);
-    if (w < SAMPLE_CHARS && bits <= 64) count_agreeing(keys, bits, &out->pairs[w], &out->triples[w]);
+    if (taken && w < SAMPLE_CHARS && bits <= 64)
+      count_agreeing(keys, bits, &out->pairs[w], &out->triples[w]);
   } else {
     count_bytes(a, s_hist, blockIdx.x - a.sample_blocks, gridDim.x - a.sample_blocks);
   }
